@@ -1,7 +1,7 @@
 """Build the sspcg CUDA library in-tree for sm_103a.
 
-Each ``csrc/*.cu`` file compiles to an object in parallel; the objects link
-into ``_lib/libsspcg.so`` (CUDA runtime linked statically).  Rebuilds only
+Each ``csrc/*.cu`` file compiles to an object in parallel (``pcg_nx.cu``
+once per state size nx); the objects link into ``_lib/libsspcg.so`` (CUDA runtime linked statically).  Rebuilds only
 when a source or header is newer than the library.
 """
 from __future__ import annotations
@@ -28,8 +28,23 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found: the sspcg CUDA library cannot be built")
 
 
+MAX_NX = 28  # SSPCG_MAX_NX
+
+
 def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+
+
+def units():
+    """(source, object name, extra flags) of every compilation, the longest first."""
+    out = []
+    for src in sources():
+        name = os.path.basename(src)[:-3]
+        if name == "pcg_nx":
+            out = [(src, f"{name}{n}", [f"-DSSPCG_NX={n}"]) for n in range(MAX_NX, 0, -1)] + out
+        else:
+            out.append((src, name, []))
+    return out
 
 
 def _newest_input() -> float:
@@ -45,20 +60,21 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
     nvcc = _nvcc()
     objdir = os.path.join(LIBDIR, "obj")
     os.makedirs(objdir, exist_ok=True)
-    jobs = jobs or max(1, min(len(sources()), os.cpu_count() or 1))
+    jobs = jobs or max(1, min(len(units()), os.cpu_count() or 1))
 
-    def compile_one(src):
-        obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
-        cmd = [nvcc, *ARCH, *FLAGS, "-c", src, "-o", obj]
+    def compile_one(unit):
+        src, name, extra = unit
+        obj = os.path.join(objdir, name + ".o")
+        cmd = [nvcc, *ARCH, *FLAGS, *extra, "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
-            raise RuntimeError(f"nvcc failed on {os.path.basename(src)}:\n{r.stderr}")
+            raise RuntimeError(f"nvcc failed on {name}:\n{r.stderr}")
         if verbose and r.stderr:
             print(r.stderr)
         return obj
 
     with cf.ThreadPoolExecutor(jobs) as ex:
-        objs = list(ex.map(compile_one, sources()))
+        objs = list(ex.map(compile_one, units()))
     tmp = LIB + f".{os.getpid()}.tmp"
     cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -84,6 +84,18 @@ int auto_block(int64_t rows) {
   return (int)std::min<int64_t>(512, std::max<int64_t>(64, t));
 }
 
+// Threads per CTA with a thread per row pair (pcg_one.cuh).
+int one_block(int64_t N, int nx) { return (int)std::max<int64_t>(64, round_up((N + 1) * tile_half(nx), 32)); }
+
+// Whether a problem runs with a thread per row pair: a solve of these options, not streaming by request, that fits
+// whole with at most 512 pairs (the registers of a thread allow no more).  Measured faster at every size it takes,
+// from 1.4x (nx = 14, N = 64) to 1.8x (nx = 4, N = 64); the line lies at what fits.
+bool one_fits(int op, const sspcg_options *o, bool f64, int64_t N, int nx, int nu) {
+  return o->schedule != SSPCG_SCHED_STREAM &&
+         pcg_one_ok(op, f64, red_mode(o->reduction), o->poly_degree, o->cg_variant,
+                    o->block_threads > 0 ? o->block_threads : 512, smem_budget(), N, nx, nu);
+}
+
 // Staged block rows K and dynamic shared memory (bytes) of a PCG problem
 // under a schedule; false when even the vectors do not fit.
 // cg: the options ask for single-reduction PCG, which the QP-form FP32 launches run (two more vectors).
@@ -136,6 +148,8 @@ namespace host {
 int sms() { return device_sms(); }
 int reduction_mode(int32_t r) { return red_mode(r); }
 int block_for_rows(int64_t rows) { return auto_block(rows); }
+int block_for_pairs(int64_t N, int nx) { return one_block(N, nx); }
+bool fits_one(int op, const sspcg_options *o, int64_t N, int nx, int nu) { return one_fits(op, o, false, N, nx, nu); }
 bool fit(int op, int sched, int N, int nx, int nu, bool f64, int poly, int cg, int *K, int64_t *bytes) {
   return pcg_fit(op, sched, N, nx, nu, f64, poly, cg, K, bytes);
 }
@@ -162,6 +176,7 @@ struct PcgGroup {
   bool gvec = false;         // vectors in a global workspace (slot_elems per CTA from scratch_off)
   bool stream = false;       // stage no block rows (the schedule option, or the tuner's choice)
   int share = 1;             // partially staged groups: stage into 1/share of the shared memory (tuner's choice)
+  bool one = false;          // a thread per row pair (one_fits for every member)
   int warps = 0;             // > 0: one problem per warp, this many warps per CTA (tuner's choice; see warp_ok)
   bool tuned = false;        // block and residency from the tuner (this plan's, or its cache)
   int64_t slot_elems = 0, scratch_off = 0;
@@ -310,14 +325,14 @@ void plan_free(sspcg_plan *p) {
 }
 
 // Tuning cache: the block size and residency the tuner picked, per (operator form, precision, reduction,
-// polynomial degree, PCG variant, nx, residency class, bucket of the group's largest N).  Process-wide; plans
+// polynomial degree, PCG variant, nx, residency class, a thread per row pair or not, bucket of the group's largest N).  Process-wide; plans
 // created after a tuning run take its choices for groups with the same key.
 struct TuneKey {
-  int set, op, f64, red, poly, cg, nx, cls, nbucket;
+  int set, op, f64, red, poly, cg, nx, cls, one, nbucket;
   bool operator<(const TuneKey &o) const {
-    const int a[9] = {set, op, f64, red, poly, cg, nx, cls, nbucket};
-    const int b[9] = {o.set, o.op, o.f64, o.red, o.poly, o.cg, o.nx, o.cls, o.nbucket};
-    return std::lexicographical_compare(a, a + 9, b, b + 9);
+    const int a[10] = {set, op, f64, red, poly, cg, nx, cls, one, nbucket};
+    const int b[10] = {o.set, o.op, o.f64, o.red, o.poly, o.cg, o.nx, o.cls, o.one, o.nbucket};
+    return std::lexicographical_compare(a, a + 10, b, b + 10);
   }
 };
 struct TuneChoice {
@@ -337,7 +352,7 @@ int n_bucket(int32_t maxN) {
 
 TuneKey tune_key(const sspcg_plan *p, const GroupSet &set, const PcgGroup &g) {
   return TuneKey{set.id, set.op, set.f64 ? 1 : 0, set.f64 ? kRedF64 : red_mode(p->opts.reduction), p->opts.poly_degree,
-                 (p->opts.cg_variant && set.op == kOpQp && !set.f64) ? 1 : 0, g.nx, g.cls, n_bucket(g.maxN)};
+                 (p->opts.cg_variant && set.op == kOpQp && !set.f64) ? 1 : 0, g.nx, g.cls, g.one ? 1 : 0, n_bucket(g.maxN)};
 }
 
 // One problem per warp exists for fully staged groups of the QP form with textbook PCG: the FP64 path, and
@@ -360,6 +375,8 @@ sspcg_status shape_group(const sspcg_plan *p, const GroupSet &set, PcgGroup &g, 
     int64_t b = 0;
     if (g.gvec) {
       b = gvec_slot(set.op, d.N, d.nx, d.nu, p->opts.poly_degree, cg);
+    } else if (g.one && g.warps == 0) {
+      b = pcg_one_layout(set.op, d.N, d.nx, d.nu).total * (int64_t)sizeof(float);
     } else {
       const int sched = g.stream ? SSPCG_SCHED_STREAM : p->opts.schedule;
       if (!pcg_fit(set.op, sched, d.N, d.nx, d.nu, set.f64, p->opts.poly_degree, cg, &K, &b, g.stream ? 1 : g.share))
@@ -373,15 +390,15 @@ sspcg_status shape_group(const sspcg_plan *p, const GroupSet &set, PcgGroup &g, 
     const int64_t slot = round_up(maxbytes, 16);
     if (slot * g.warps > smem_budget()) return SSPCG_ERR_UNSUPPORTED;
     g.block = 32 * g.warps;
-    cudaError_t e = occupancy_pcg(g.nx, set.op, red, set.f64, false, cgv, true, g.block, (size_t)(slot * g.warps),
-                                  &ctas);
+    cudaError_t e = occupancy_pcg(g.nx, set.op, red, set.f64, false, cgv, true, false, g.block,
+                                  (size_t)(slot * g.warps), &ctas);
     if (e != cudaSuccess) return cuda_fail(e);
     if (ctas < 1) return SSPCG_ERR_UNSUPPORTED;
     g.smem = (size_t)(slot * g.warps);
     g.grid = (int)std::min<int64_t>((g.nwork + g.warps - 1) / g.warps, (int64_t)ctas * device_sms());
     return SSPCG_OK;
   }
-  cudaError_t e = occupancy_pcg(g.nx, set.op, red, set.f64, g.gvec, cgv, false, g.block,
+  cudaError_t e = occupancy_pcg(g.nx, set.op, red, set.f64, g.gvec, cgv, false, g.one, g.block,
                                 g.gvec ? 0 : (size_t)maxbytes, &ctas);
   if (e != cudaSuccess) return cuda_fail(e);
   ctas = std::max(1, ctas);
@@ -404,20 +421,25 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
   // class 0: not fully resident (takes the whole budget); classes 1..3: fully resident within
   // budget/2, /4, /8 (several CTAs per SM); class 4: the rest of the fully resident problems
   // class 5: vectors in a global workspace (they alone exceed the shared memory)
+  // each class split into the problems that run with a thread per row pair and the others
   constexpr int kClasses = 6;
-  std::vector<std::vector<int32_t>> buckets(kClasses * (kMaxNx + 1));
+  std::vector<std::vector<int32_t>> buckets(2 * kClasses * (kMaxNx + 1));
   std::vector<int64_t> bytes(descs.size(), 0);
   const int64_t budget = smem_budget();
   for (int32_t i : members) {
     const ProbDesc &d = descs[i];
     int K = 0;
-    if (!pcg_fit(set.op, p->opts.schedule, d.N, d.nx, d.nu, set.f64, p->opts.poly_degree, p->opts.cg_variant, &K,
-                 &bytes[i])) {
+    const bool one = one_fits(set.op, &p->opts, set.f64, d.N, d.nx, d.nu);
+    if (one) {
+      K = d.N + 1;
+      bytes[i] = pcg_one_layout(set.op, d.N, d.nx, d.nu).total * (int64_t)sizeof(float);
+    } else if (!pcg_fit(set.op, p->opts.schedule, d.N, d.nx, d.nu, set.f64, p->opts.poly_degree, p->opts.cg_variant, &K,
+                        &bytes[i])) {
       if (set.op != kOpQp) {  // global-vector kernels exist for the QP operator form only
         set.unsupported = true;
         continue;
       }
-      buckets[kClasses * d.nx + 5].push_back(i);
+      buckets[2 * (kClasses * d.nx + 5)].push_back(i);
       continue;
     }
     int cls = 0;
@@ -425,11 +447,12 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
       const int64_t need = bytes[i] + kPcgStaticSmem + 1024;
       cls = need * 8 <= budget ? 3 : need * 4 <= budget ? 2 : need * 2 <= budget ? 1 : 4;
     }
-    buckets[kClasses * d.nx + cls].push_back(i);
+    buckets[2 * (kClasses * d.nx + cls) + (one ? 1 : 0)].push_back(i);
   }
   for (int nx = 1; nx <= kMaxNx; ++nx) {
-    for (int r = 0; r < kClasses; ++r) {
-      auto &b = buckets[kClasses * nx + r];
+    for (int rb = 0; rb < 2 * kClasses; ++rb) {
+      const int r = rb / 2;
+      auto &b = buckets[2 * kClasses * nx + rb];
       if (b.empty()) continue;
       std::stable_sort(b.begin(), b.end(), [&](int32_t x, int32_t y) { return descs[x].N > descs[y].N; });
       PcgGroup g;
@@ -437,6 +460,7 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
       g.cls = r;
       g.resident = r != 0 && r != 5;
       g.gvec = r == 5;
+      g.one = rb % 2 == 1;
       g.f64 = set.f64;
       g.stream = p->opts.schedule == SSPCG_SCHED_STREAM;
       g.members = b;
@@ -447,13 +471,13 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
         // bytes per iteration times iterations, which grow about as sqrt(N + 1)
         g.work += std::pow((double)(d.N + 1), 1.5) * d.nx * (3.0 * d.nx + d.nu);
       }
-      g.block = p->opts.block_threads > 0 ? p->opts.block_threads : auto_block(g.maxrows);
+      g.block = p->opts.block_threads > 0 ? p->opts.block_threads : g.one ? one_block(g.maxN, nx) : auto_block(g.maxrows);
       g.nwork = (int32_t)b.size();
       if (p->opts.block_threads == 0 && p->opts.schedule == SSPCG_SCHED_AUTO) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(tune_key(p, set, g));
         if (it != g_tune_cache.end()) {
-          g.block = it->second.block;
+          if (!g.one) g.block = it->second.block;  // with a thread per row pair the problems set the block size
           g.stream = it->second.stream && r == 0;
           g.share = r == 0 ? it->second.share : 1;
           g.warps = warp_ok(p, set, g) ? it->second.warps : 0;
@@ -463,7 +487,14 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
       if (p->opts.schedule == SSPCG_SCHED_WARP && warp_ok(p, set, g)) {
         // one problem per warp: as many warps (a power of two, at most 16) as slots of the largest member fit
         int64_t slot = 0;
-        for (int32_t i : b) slot = std::max(slot, round_up(bytes[i], 16));
+        for (int32_t i : b) {
+          int K = 0;
+          int64_t need = 0;
+          if (!pcg_fit(set.op, SSPCG_SCHED_RESIDENT, descs[i].N, nx, descs[i].nu, set.f64, p->opts.poly_degree,
+                       p->opts.cg_variant, &K, &need))
+            need = smem_budget();
+          slot = std::max(slot, round_up(need, 16));
+        }
         const int64_t fit = slot > 0 ? smem_budget() / slot : 1;
         g.warps = 1;
         while (g.warps < 16 && 2 * g.warps <= fit) g.warps *= 2;
@@ -479,8 +510,10 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
         set.scratch_elems += (int64_t)g.max_grid * g.slot_elems;
       }
       sspcg_status s = shape_group(p, set, g, descs);
-      if (s == SSPCG_ERR_UNSUPPORTED && g.warps > 0) {  // a cached warp count whose slots do not fit this group
+      if (s == SSPCG_ERR_UNSUPPORTED && g.warps > 0) {  // a warp count whose slots do not fit this group
         g.warps = 0;
+        if (p->opts.block_threads == 0) g.block = g.one ? one_block(g.maxN, nx) : auto_block(g.maxrows);
+        else g.block = p->opts.block_threads;
         s = shape_group(p, set, g, descs);
       }
       if (s != SSPCG_OK) return s;
@@ -553,6 +586,7 @@ sspcg_status launch_sets(sspcg_plan *p, std::initializer_list<SetLaunch> list, c
     set_gvec(a, p, *all[i].set, g);
     if (g.stream) a.max_resident = 0;
     a.warp = g.warps > 0 ? 1 : 0;
+    a.one = g.one && g.warps == 0 ? 1 : 0;
     cudaStream_t s = i == 0 ? st : p->side[i - 1];
     const int red = g.f64 ? kRedF64 : red_mode(p->opts.reduction);
     SSPCG_CUDA(launch_pcg(g.nx, all[i].set->op, red, g.f64, a, g.grid, g.block, g.smem, s));
@@ -673,7 +707,9 @@ static sspcg_status solve_single(int op, bool f64, int32_t N, int32_t nx, int32_
   if (op == kOpBlock && (!D || (N > 0 && !E))) return SSPCG_ERR_INVALID_ARG;
   int K = 0;
   int64_t bytes = 0;
-  if (!pcg_fit(op, opts->schedule, N, nx, nu, f64, opts->poly_degree, opts->cg_variant, &K, &bytes))
+  const bool one = one_fits(op, opts, f64, N, nx, nu);
+  if (one) bytes = pcg_one_layout(op, N, nx, nu).total * (int64_t)sizeof(float);
+  else if (!pcg_fit(op, opts->schedule, N, nx, nu, f64, opts->poly_degree, opts->cg_variant, &K, &bytes))
     return SSPCG_ERR_UNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
   PcgArgs a = make_args(opts);
@@ -682,7 +718,10 @@ static sspcg_status solve_single(int op, bool f64, int32_t N, int32_t nx, int32_
   a.A = A; a.B = B; a.qd = qd; a.rd = rd; a.D = D; a.E = E; a.PD = PD; a.PE = PE;
   a.gamma = gamma; a.lambda = lambda; a.iters = iters; a.relres = relres; a.status = status;
   a.lambda_f32 = f64 ? 0 : 1;
-  const int block = opts->block_threads > 0 ? opts->block_threads : auto_block((int64_t)(N + 1) * nx);
+  a.one = one ? 1 : 0;
+  const int block = opts->block_threads > 0 ? opts->block_threads
+                    : one                   ? one_block(N, nx)
+                                            : auto_block((int64_t)(N + 1) * nx);
   SSPCG_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
   SSPCG_CUDA(launch_pcg(nx, op, f64 ? kRedF64 : red_mode(opts->reduction), f64, a, 1, block, (size_t)bytes, st));
   return SSPCG_OK;
@@ -1224,6 +1263,7 @@ sspcg_status time_group(sspcg_plan *p, const GroupSet &set, const PcgGroup &g, c
   set_gvec(a, p, set, g);
   if (g.stream) a.max_resident = 0;
   a.warp = g.warps > 0 ? 1 : 0;
+  a.one = g.one && g.warps == 0 ? 1 : 0;
   const int red = g.f64 ? kRedF64 : red_mode(p->opts.reduction);
   float best = 1e30f;
   for (int rep = 0; rep < 3; ++rep) {
@@ -1255,13 +1295,14 @@ sspcg_status tune_set(sspcg_plan *p, GroupSet &set, const std::vector<ProbDesc> 
     // from at most 16 rows per thread to at most one
     const int64_t max_block = std::max<int64_t>(64, round_up(g.maxrows, 32));
     const int64_t min_block = std::min<int64_t>(max_block, g.maxrows / 16);
+    // (with a thread per row pair, the group's own block size)
     // residency candidates: partially staged groups may stage into 1/2 .. 1/4 of the shared memory (several
     // CTAs per SM) or stream every block row; the other classes keep their staging
     for (int cand = 0; cand < (g.cls == 0 ? 5 : 1); ++cand) {
       const bool stream = cand == 4;
       const int share = cand < 4 ? cand + 1 : 1;
       for (int blk : kBlocks) {
-        if (blk > max_block || blk < min_block ||
+        if (g.one || blk > max_block || blk < min_block ||
             (blk == orig.block && stream == orig.stream && share == orig.share))
           continue;
         PcgGroup c = orig;

@@ -99,6 +99,45 @@ __host__ __device__ inline int pcg_max_resident(int op, int N, int nx, int nu, i
   return lo;
 }
 
+// The kernel with a thread per row pair (pcg_one.cuh): FP32 textbook PCG with double-float sums and a degree-0
+// preconditioner, for problems that fit in shared memory whole.
+//
+// Its blocks are staged as 2 x 2 tiles: tile (q, c) holds rows 2q, 2q+1 and columns 2c, 2c+1 as four consecutive
+// values (m00, m01, m10, m11), zero past an odd last row or column.  A thread owns a pair of rows of the unknowns,
+// so one 128-bit load feeds four multiply-adds whichever way the block is read: along tile row q for rows 2q, 2q+1
+// of M v, or down tile column c for rows 2c, 2c+1 of M^T v.  Tile rows are an odd number of tiles long, so that
+// eight threads on consecutive tile rows (one phase of a 128-bit shared-memory load) touch 32 distinct banks.
+__host__ __device__ __forceinline__ int tile_half(int x) { return (x + 1) >> 1; }
+__host__ __device__ __forceinline__ int tile_ld(int cols) { return tile_half(cols) | 1; }
+__host__ __device__ __forceinline__ int tile_block(int rows, int cols) {  // values of a block
+  return cols > 0 ? 4 * tile_half(rows) * tile_ld(cols) : 0;
+}
+
+// Its shared memory, in floats; regions and vectors as in PcgLayout, without w and x.  A single-knot problem
+// (N = 0) has one zero off-diagonal slot of each kind.
+struct OneLayout {
+  int64_t p, r, v, vu, iq, ir, m0, m1, pd, pe, total;
+};
+__host__ __device__ inline OneLayout pcg_one_layout(int op, int N, int nx, int nu) {
+  OneLayout L{};
+  const int64_t n = N + 1, NXP = vec_stride(nx), NUP = vec_stride(nu), RVP = (n + 2) * NXP;
+  const int64_t blk = tile_block(nx, nx), blkb = tile_block(nx, nu), slots = N > 0 ? N : 1;
+  const bool qp = op == kOpQp;
+  int64_t o = 0;
+  L.p = o + NXP; o += RVP;
+  L.r = o + NXP; o += RVP;
+  L.v = o + NXP; o += qp ? RVP : 0;
+  L.vu = o + NUP; o += qp ? n * NUP : 0;  // v_u(-1) is zero
+  L.iq = o; o += qp ? n * NXP : 0;
+  L.ir = o; o += qp ? N * NUP : 0;
+  L.m0 = o; o += qp ? slots * blk : n * blk;  // A_k; D_k, transposed
+  L.m1 = o; o += slots * (qp ? blkb : blk);   // B_k; E_k
+  L.pd = o; o += n * blk;                     // PD_k, transposed
+  L.pe = o; o += slots * blk;                 // PE_k
+  L.total = o;
+  return L;
+}
+
 // Arguments of a PCG launch (by value).
 struct PcgArgs {
   ProbSet ps;
@@ -124,6 +163,7 @@ struct PcgArgs {
   void *gscratch;        // vectors in global memory: CTA b uses gscratch + b * gstride elements
   int64_t gstride;       //   (nullptr: vectors in shared memory)
   int32_t warp;          // 1: one problem per warp (smem_elems per warp), QP form, textbook PCG
+  int32_t one;           // 1: the kernel with a thread per row pair (pcg_one_ok holds for every problem)
   const float *pad;      // padded copies of A, B, PE of the streamed problems (QP form, FP32), or nullptr
   const int64_t *pad_off;  // per problem id: offset of its copies in pad, or -1 (read the inputs)
 };
@@ -151,9 +191,17 @@ cudaError_t launch_pcg(int nx, int op, int red, bool f64, const PcgArgs &a, int 
 int pcg_max_smem_bytes();
 // CTAs of that PCG variant that fit on one SM at ``block`` threads and ``smem`` bytes of dynamic shared memory
 // (registers, threads and shared memory; gv: vectors in a global workspace; cg: single-reduction PCG;
-// warp: one problem per warp).
-cudaError_t occupancy_pcg(int nx, int op, int red, bool f64, bool gv, bool cg, bool warp, int block, size_t smem,
-                          int *ctas);
+// warp: one problem per warp; one: a thread per row pair).
+cudaError_t occupancy_pcg(int nx, int op, int red, bool f64, bool gv, bool cg, bool warp, bool one, int block,
+                          size_t smem, int *ctas);
+
+// Whether the kernel with a thread per row pair solves a problem of these options in a CTA of ``block`` threads
+// with ``budget`` bytes of dynamic shared memory.
+inline bool pcg_one_ok(int op, bool f64, int red, int poly, int cg, int block, int64_t budget, int64_t N, int nx,
+                       int nu) {
+  return !f64 && red == kRedDf && poly == 0 && !(cg && op == kOpQp) && (N + 1) * tile_half(nx) <= block &&
+         pcg_one_layout(op, (int)N, nx, nu).total * (int64_t)sizeof(float) <= budget;
+}
 
 // Schur build and preconditioner assembly; Real = float (FP32 blocks) or
 // double (the FP64 path).  refs[i] = (problem, block row) of work item i

@@ -24,6 +24,8 @@ namespace host {  // defined in api.cu
 int sms();
 int reduction_mode(int32_t r);
 int block_for_rows(int64_t rows);
+int block_for_pairs(int64_t N, int nx);
+bool fits_one(int op, const sspcg_options *o, int64_t N, int nx, int nu);
 bool fit(int op, int sched, int N, int nx, int nu, bool f64, int poly, int cg, int *K, int64_t *bytes);
 sspcg_status check_options(const sspcg_options *o);
 bool valid_shape(int N, int nx, int nu);
@@ -175,7 +177,8 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
   s.nprob = nprob;
   struct Group {
     int32_t count = 0, first = 0;
-    int64_t rows = 0, smem = 0;
+    int64_t rows = 0, smem = 0, maxN = 0, smem_one = 0;
+    bool one = true;  // every problem of the group runs with a thread per row pair
   } groups[kMaxNx + 1];
   for (int32_t i = 0; i < nprob; ++i) {
     s.N[i] = (int16_t)N[i];
@@ -183,10 +186,15 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
     s.nu[i] = (uint8_t)nu[i];
     int K = 0;
     int64_t bytes = 0;
+    Group &g = groups[nx[i]];
+    const bool one = host::fits_one(kOpQp, opts, N[i], nx[i], nu[i]);
     if (!host::fit(kOpQp, opts->schedule, N[i], nx[i], nu[i], false, opts->poly_degree, opts->cg_variant, &K,
                    &bytes))
       return SSPCG_ERR_UNSUPPORTED;
-    Group &g = groups[nx[i]];
+    g.one = g.one && one;
+    if (one)
+      g.smem_one = std::max(g.smem_one, pcg_one_layout(kOpQp, N[i], nx[i], nu[i]).total * (int64_t)sizeof(float));
+    g.maxN = std::max<int64_t>(g.maxN, N[i]);
     ++g.count;
     g.rows = std::max<int64_t>(g.rows, (int64_t)(N[i] + 1) * nx[i]);
     g.smem = std::max<int64_t>(g.smem, bytes);
@@ -230,15 +238,19 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
   for (int m = 1; m <= kMaxNx; ++m) {
     const Group &g = groups[m];
     if (g.count == 0) continue;
-    const int block = opts->block_threads > 0 ? opts->block_threads : host::block_for_rows(g.rows);
-    const int by_smem = (int)std::max<int64_t>(1, (228 * 1024) / (g.smem + 2048));
+    const int block = opts->block_threads > 0 ? opts->block_threads
+                      : g.one                 ? host::block_for_pairs(g.maxN, m)
+                                              : host::block_for_rows(g.rows);
+    const int64_t smem = g.one ? g.smem_one : g.smem;
+    const int by_smem = (int)std::max<int64_t>(1, (228 * 1024) / (smem + 2048));
     const int by_thr = std::max(1, 2048 / block);
     const int grid = (int)std::min<int64_t>(g.count, (int64_t)std::min(by_smem, by_thr) * host::sms());
     PcgArgs ga = a;
     ga.work = scr->work + g.first;
     ga.nwork = g.count;
     ga.counter = scr->counters + counter++;
-    e = launch_pcg(m, kOpQp, host::reduction_mode(opts->reduction), false, ga, grid, block, (size_t)g.smem, st);
+    ga.one = g.one ? 1 : 0;
+    e = launch_pcg(m, kOpQp, host::reduction_mode(opts->reduction), false, ga, grid, block, (size_t)smem, st);
     if (e != cudaSuccess) return host::cuda_error(e);
   }
   return SSPCG_OK;
