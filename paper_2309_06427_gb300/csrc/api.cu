@@ -220,6 +220,7 @@ struct NxGroup {
 struct sspcg_plan {
   int32_t nprob = 0;
   int mx = 1;       // largest nx and nu of the batch
+  int32_t max_nu = 0, max_N = 0;
   int mx_tiny = 1;  // of its FP64 subset
   std::vector<NxGroup> nxg_all, nxg_tiny;
   sspcg_options opts{};
@@ -228,6 +229,7 @@ struct sspcg_plan {
   int64_t sizes[SSPCG_NUM_ARRAYS] = {};
   ProbDesc *d_desc = nullptr;
   int2 *d_kref = nullptr, *d_oref = nullptr;  // (problem, block row) per knot / off-diagonal block
+  int32_t *d_order = nullptr;  // problems, those with the most matrix entries first
   int64_t total_knots = 0, total_off = 0;
   std::vector<int64_t> knot_start;      // first knot (index into d_kref) of each problem, nprob + 1 entries
   int64_t *d_knot_start = nullptr;
@@ -288,7 +290,7 @@ namespace {
 void plan_free(sspcg_plan *p) {
   if (!p) return;
   if (p->graph) cudaGraphExecDestroy(p->graph);
-  for (void *ptr : {(void *)p->d_desc, (void *)p->d_kref, (void *)p->d_oref, (void *)p->d_knot_start, (void *)p->d_tdesc,
+  for (void *ptr : {(void *)p->d_desc, (void *)p->d_kref, (void *)p->d_oref, (void *)p->d_order, (void *)p->d_knot_start, (void *)p->d_tdesc,
                     (void *)p->d_tkref, (void *)p->d_toref, (void *)p->D64, (void *)p->E64,
                     (void *)p->PD64, (void *)p->PE64, (void *)p->d_work, (void *)p->d_counters, (void *)p->d_scratch, (void *)p->hbuf,
                     (void *)p->hint, (void *)p->hdbl, (void *)p->d_pad, (void *)p->d_pad_off, (void *)p->d_pad_list})
@@ -756,7 +758,7 @@ sspcg_status sspcg_residual_qp(int32_t N, int32_t nx, int32_t nu, const float *A
   if (!shape_ok(N, nx, nu) || !qd || !gamma || !lambda || !relres_true) return SSPCG_ERR_INVALID_ARG;
   if (N > 0 && (!A || !rd || (nu > 0 && !B))) return SSPCG_ERR_INVALID_ARG;
   ProbSet ps{nullptr, single_desc(N, nx, nu), 1};
-  SSPCG_CUDA(launch_residual_qp(ps, A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
+  SSPCG_CUDA(launch_residual_qp(ps, nullptr, A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
   return SSPCG_OK;
 }
 
@@ -799,6 +801,8 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     off_start[i + 1] = off_start[i] + Ni;
     all.push_back(i);
     p->mx = std::max(p->mx, std::max(nx[i], nu[i]));
+    p->max_nu = std::max(p->max_nu, nu[i]);
+    p->max_N = std::max(p->max_N, N[i]);
     const bool f64 = opts->precision == SSPCG_PRECISION_F64 ||
                      (opts->precision == SSPCG_PRECISION_AUTO && n * m <= kTinyUnknowns);
     (f64 ? tiny : main_set).push_back(i);
@@ -831,6 +835,12 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     if ((e = upload(&p->d_kref, row_refs(p->hdesc, 0))) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = upload(&p->d_oref, row_refs(p->hdesc, 1))) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = upload(&p->d_knot_start, p->knot_start)) != cudaSuccess) return fail(cuda_fail(e));
+    std::vector<int32_t> order(all);
+    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+      auto entries = [&](const ProbDesc &d) { return (int64_t)(d.N + 1) * d.nx * (d.nx + d.nu); };
+      return entries(p->hdesc[x]) > entries(p->hdesc[y]);
+    });
+    if ((e = upload(&p->d_order, order)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = make_nx_groups(p->hdesc, all, p->nxg_all)) != cudaSuccess) return fail(cuda_fail(e));
     if (p->ntiny > 0) {
       std::vector<int32_t> tl(p->ntiny);
@@ -1145,7 +1155,7 @@ sspcg_status sspcg_residual_qp_batched(sspcg_plan *plan, const float *A, const f
   if (plan->nprob == 0) return SSPCG_OK;
   if (!qd || !gamma || !lambda || !relres_true || (plan->total_off > 0 && (!A || !B || !rd)))
     return SSPCG_ERR_INVALID_ARG;
-  SSPCG_CUDA(launch_residual_qp(plan_set(plan), A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
+  SSPCG_CUDA(launch_residual_qp(plan_set(plan), plan->d_order, A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
   return SSPCG_OK;
 }
 
@@ -1583,8 +1593,8 @@ PlanView plan_view(const sspcg_plan *p) {
   v.knot_start = p->knot_start.data();
   v.d_knot_start = p->d_knot_start;
   v.total_off = p->total_off;
-  v.max_nu = 0;
-  for (const ProbDesc &d : p->hdesc) v.max_nu = std::max(v.max_nu, d.nu);
+  v.max_nu = p->max_nu;
+  v.max_N = p->max_N;
   return v;
 }
 sspcg_status build_half(sspcg_plan *plan, sspcg_precond kind, const float *A, const float *B, const float *qd,

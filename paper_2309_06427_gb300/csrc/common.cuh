@@ -134,6 +134,45 @@ __device__ __forceinline__ df df_sqrt(df x) {
 __host__ __device__ __forceinline__ int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ __forceinline__ int64_t round_up(int64_t a, int64_t b) { return cdiv(a, b) * b; }
 
+// Chunks of consecutive block rows of one problem, for kernels that give a thread one column of a chunk's [A_k B_k]
+// (or one row of it): as many block rows as make kChunkItems columns.  kChunkFloats holds a chunk's blocks with odd
+// row strides for every nx, nu <= 28 (the most is 7616, at nx = 28, nu = 4).
+constexpr int kChunkItems = 256;
+constexpr int kChunkFloats = 7616;
+__host__ __device__ __forceinline__ int chunk_rows(int nx, int nu) {
+  const int c = kChunkItems / (nx + nu);
+  return c > 64 ? 64 : c;
+}
+
+// Quotients by a divisor d <= 64 known at run time, for e < 2^20: the high word of e times ceil(2^32 / d), whose
+// excess over e / d is below e d / 2^32 < 1 / d.
+struct Divisor {
+  uint32_t mul;  // 0: d = 1
+  __device__ __forceinline__ explicit Divisor(int d) : mul(d > 1 ? 0xffffffffu / (uint32_t)d + 1u : 0u) {}
+  __device__ __forceinline__ int quotient(int e) const { return mul ? (int)__umulhi((uint32_t)e, mul) : e; }
+};
+
+// f(e, src[e]) for e < n, consecutive threads on consecutive values, eight loads of a thread in flight at a time
+// (chunks are short: with the loads one after the other, waiting for them is most of the time).
+template <typename F>
+__device__ __forceinline__ void for_values(const float *src, int n, int tid, int nthr, F &&f) {
+  constexpr int U = 8;
+  for (int e0 = tid; e0 < n; e0 += U * nthr) {
+    float v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = e0 + u * nthr < n ? __ldg(src + e0 + u * nthr) : 0.0f;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (e0 + u * nthr < n) f(e0 + u * nthr, v[u]);
+  }
+}
+
+// ``rows`` dense rows of width w (global) into rows of stride ld (shared memory).
+__device__ __forceinline__ void stage_chunk(float *dst, const float *src, int rows, int w, int ld, int tid, int nthr) {
+  const Divisor by_w(w);
+  for_values(src, rows * w, tid, nthr, [&](int e, float v) { dst[e + by_w.quotient(e) * (ld - w)] = v; });
+}
+
 // Find the problem owning global knot g: knot_start is an exclusive prefix
 // of (N_i + 1) with nprob + 1 entries.
 __device__ __forceinline__ int find_problem(const int64_t *knot_start, int nprob, int64_t g) {
