@@ -211,10 +211,9 @@ struct NxGroup {
   int nx = 0;
   int mx = 1;  // largest nx and nu of the group
   int32_t nprob = 0;
-  int64_t knots = 0, offs = 0;
+  int64_t knots = 0;
   ProbDesc *d_desc = nullptr;
   int2 *d_refs = nullptr;   // (index into d_desc, block row) per knot
-  int2 *d_orefs = nullptr;  // (index into d_desc, block row) per off-diagonal block
 };
 
 struct sspcg_plan {
@@ -228,7 +227,7 @@ struct sspcg_plan {
   std::vector<int64_t> offsets[SSPCG_NUM_ARRAYS];
   int64_t sizes[SSPCG_NUM_ARRAYS] = {};
   ProbDesc *d_desc = nullptr;
-  int2 *d_kref = nullptr, *d_oref = nullptr;  // (problem, block row) per knot / off-diagonal block
+  int2 *d_kref = nullptr;  // (problem, block row) per knot
   int32_t *d_order = nullptr;  // problems, those with the most matrix entries first
   int64_t total_knots = 0, total_off = 0;
   std::vector<int64_t> knot_start;      // first knot (index into d_kref) of each problem, nprob + 1 entries
@@ -290,7 +289,7 @@ namespace {
 void plan_free(sspcg_plan *p) {
   if (!p) return;
   if (p->graph) cudaGraphExecDestroy(p->graph);
-  for (void *ptr : {(void *)p->d_desc, (void *)p->d_kref, (void *)p->d_oref, (void *)p->d_order, (void *)p->d_knot_start, (void *)p->d_tdesc,
+  for (void *ptr : {(void *)p->d_desc, (void *)p->d_kref, (void *)p->d_order, (void *)p->d_knot_start, (void *)p->d_tdesc,
                     (void *)p->d_tkref, (void *)p->d_toref, (void *)p->D64, (void *)p->E64,
                     (void *)p->PD64, (void *)p->PE64, (void *)p->d_work, (void *)p->d_counters, (void *)p->d_scratch, (void *)p->hbuf,
                     (void *)p->hint, (void *)p->hdbl, (void *)p->d_pad, (void *)p->d_pad_off, (void *)p->d_pad_list})
@@ -299,7 +298,6 @@ void plan_free(sspcg_plan *p) {
     for (NxGroup &g : *v) {
       cudaFree(g.d_desc);
       cudaFree(g.d_refs);
-      cudaFree(g.d_orefs);
     }
   for (auto &a : p->aslot) {
     cudaFree(a.buf);
@@ -315,7 +313,6 @@ void plan_free(sspcg_plan *p) {
   for (NxGroup &g : p->nxg_r) {
     cudaFree(g.d_desc);
     cudaFree(g.d_refs);
-    cudaFree(g.d_orefs);
   }
   if (p->h2d) cudaStreamDestroy(p->h2d);
   if (p->d2h) cudaStreamDestroy(p->d2h);
@@ -625,17 +622,15 @@ cudaError_t make_nx_groups(const std::vector<ProbDesc> &descs, const std::vector
     for (int32_t i : members)
       if (descs[i].nx == nx) sub.push_back(descs[i]);
     if (sub.empty()) continue;
-    const std::vector<int2> refs = row_refs(sub, 0), orefs = row_refs(sub, 1);
+    const std::vector<int2> refs = row_refs(sub, 0);
     NxGroup g;
     g.nx = nx;
     for (const ProbDesc &d : sub) g.mx = std::max(g.mx, std::max(d.nx, d.nu));
     g.nprob = (int32_t)sub.size();
     g.knots = (int64_t)refs.size();
-    g.offs = (int64_t)orefs.size();
     out.push_back(g);  // pushed first so that plan_free releases partial uploads
     cudaError_t e = upload(&out.back().d_desc, sub);
     if (e == cudaSuccess) e = upload(&out.back().d_refs, refs);
-    if (e == cudaSuccess) e = upload(&out.back().d_orefs, orefs);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -656,8 +651,7 @@ sspcg_status sspcg_build_schur(int32_t N, int32_t nx, int32_t nu, const float *A
   if (!shape_ok(N, nx, nu)) return SSPCG_ERR_INVALID_ARG;
   if (!qd || !D || (N > 0 && (!A || !rd || !E || (nu > 0 && !B)))) return SSPCG_ERR_INVALID_ARG;
   ProbSet ps{nullptr, single_desc(N, nx, nu), 1};
-  SSPCG_CUDA(launch_schur_build<float>(ps, nullptr, N + 1, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms(),
-                                       std::max(nx, nu)));
+  SSPCG_CUDA(launch_schur_f32(ps, N, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
   return SSPCG_OK;
 }
 
@@ -692,8 +686,7 @@ sspcg_status sspcg_build_precond(int32_t N, int32_t nx, sspcg_precond kind, cons
   ProbSet ps{nullptr, single_desc(N, nx, 0), 1};
   SSPCG_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
   SSPCG_CUDA(launch_precond_inv<float>(ps, nullptr, N + 1, nx, (int)kind, D, PD, status, st));
-  SSPCG_CUDA(
-      launch_precond_off<float>(ps, nullptr, N, (int)kind, E, PD, PE, st, device_sms(), (int64_t)N * nx * nx, nx));
+  SSPCG_CUDA(launch_precond_off_f32(ps, N, (int)kind, E, PD, PE, st, device_sms(), (int64_t)N * nx * nx));
   return SSPCG_OK;
 }
 
@@ -833,7 +826,6 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     cudaError_t e;
     if ((e = upload(&p->d_desc, p->hdesc)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = upload(&p->d_kref, row_refs(p->hdesc, 0))) != cudaSuccess) return fail(cuda_fail(e));
-    if ((e = upload(&p->d_oref, row_refs(p->hdesc, 1))) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = upload(&p->d_knot_start, p->knot_start)) != cudaSuccess) return fail(cuda_fail(e));
     std::vector<int32_t> order(all);
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
@@ -981,8 +973,7 @@ sspcg_status sspcg_build_schur_batched(sspcg_plan *plan, const float *A, const f
   if (plan->nprob == 0) return SSPCG_OK;
   if (!qd || !D || !aligned16(qd) || !aligned16(D)) return SSPCG_ERR_INVALID_ARG;
   if (plan->total_off > 0 && (!A || !rd || !E || !B)) return SSPCG_ERR_INVALID_ARG;
-  SSPCG_CUDA(launch_schur_build<float>(plan_set(plan), plan->d_kref, plan->total_knots, A, B, qd, rd, D, E,
-                                       (cudaStream_t)stream, device_sms(), plan->mx));
+  SSPCG_CUDA(launch_schur_f32(plan_set(plan), plan->max_N, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
   return SSPCG_OK;
 }
 
@@ -1071,8 +1062,8 @@ sspcg_status sspcg_build_precond_batched(sspcg_plan *plan, sspcg_precond kind, c
   for (const NxGroup &g : plan->nxg_all)
     SSPCG_CUDA(launch_precond_inv<float>(ProbSet{g.d_desc, ProbDesc{}, g.nprob}, g.d_refs, g.knots, g.nx,
                                          (int)kind, D, PD, status, st));
-  SSPCG_CUDA(launch_precond_off<float>(plan_set(plan), plan->d_oref, plan->total_off, (int)kind, E, PD, PE, st,
-                                       device_sms(), plan->sizes[SSPCG_ARRAY_OFF], plan->mx));
+  SSPCG_CUDA(launch_precond_off_f32(plan_set(plan), plan->max_N, (int)kind, E, PD, PE, st, device_sms(),
+                                    plan->sizes[SSPCG_ARRAY_OFF]));
   return SSPCG_OK;
 }
 

@@ -1,6 +1,8 @@
 // Schur-block build (Sec. II-A) and preconditioner assembly (Eq. stair_inv,
 // Sec. III, Sec. IV, Eq. jacobi).  One warp per knot; the batch is a flat
-// list of knots whose (problem, block row) pairs the plan tabulates.
+// list of knots whose (problem, block row) pairs the plan tabulates.  The FP32
+// Schur blocks of diagonal costs and FP32 off-diagonal blocks are in
+// build_f32.cu; here these two run for the FP64 path.
 #include <algorithm>
 #include <type_traits>
 
@@ -532,9 +534,6 @@ cudaError_t launch_precond_off(const ProbSet &ps, const int2 *refs, int64_t tota
   return cudaGetLastError();
 }
 
-template cudaError_t launch_schur_build<float>(const ProbSet &, const int2 *, int64_t, const float *, const float *,
-                                               const float *, const float *, float *, float *, cudaStream_t, int,
-                                               int);
 template cudaError_t launch_schur_build<double>(const ProbSet &, const int2 *, int64_t, const float *,
                                                 const float *, const float *, const float *, double *, double *,
                                                 cudaStream_t, int, int);
@@ -542,8 +541,6 @@ template cudaError_t launch_precond_inv<float>(const ProbSet &, const int2 *, in
                                                float *, int32_t *, cudaStream_t);
 template cudaError_t launch_precond_inv<double>(const ProbSet &, const int2 *, int64_t, int, int, const double *,
                                                 double *, int32_t *, cudaStream_t);
-template cudaError_t launch_precond_off<float>(const ProbSet &, const int2 *, int64_t, int, const float *,
-                                               const float *, float *, cudaStream_t, int, int64_t, int);
 template cudaError_t launch_precond_off<double>(const ProbSet &, const int2 *, int64_t, int, const double *,
                                                 const double *, double *, cudaStream_t, int, int64_t, int);
 
