@@ -58,13 +58,11 @@ cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, 
                               bf16 *Cb, float *Cf, int *err, cudaStream_t st);
 // False when the driver's tensor-map encoder is unavailable.
 bool tc_available();
-// part[s][N1][N2] = sum over rows m of split s of G[m][n1] X[m][n2].
+// part[s kParams + n1 N2 + n2] = sum over rows m of split s of G[m][n1] X[m][n2].
 cudaError_t launch_gemm_tn(const bf16 *G, int N1, const bf16 *X, int N2, int64_t M, float *part, cudaStream_t st);
 int64_t gemm_tn_splits(int64_t M);
-// part[chunk][N] = column sums of Y[M][N] over the same row chunks as launch_gemm_tn.
-cudaError_t launch_colsum(const bf16 *Y, int64_t M, int N, float *part, cudaStream_t st);
-// out[i] = sum_s part[s][i], s in order.
-cudaError_t launch_reduce_splits(const float *part, int64_t splits, int64_t n, float *out, cudaStream_t st);
+// part[s kParams + kB3, kB2, kB1 + c] = column sums of dY [M][kOut], dH2 and dH1 [M][kHid] over the same row chunks.
+cudaError_t launch_colsum(const bf16 *dY, const bf16 *dH2, const bf16 *dH1, int64_t M, float *part, cudaStream_t st);
 
 // S^2-norm loss of problems [p0, p1) whose rows start at knot_start[p] - row0 in Y/U/dY.
 struct LossArgs {
@@ -79,10 +77,12 @@ struct LossArgs {
 };
 cudaError_t launch_loss(const LossArgs &a, cudaStream_t st);
 
-// Adam on the flat parameters (update = false: only refresh the bf16 copies).
+// Adam on the flat parameters from the splits of their gradients, whose sums go to g (update = false: only refresh the
+// bf16 copies).
 struct AdamArgs {
-  float *w, *m, *v;
-  const float *g;
+  float *w, *m, *v, *g;
+  const float *part;
+  int64_t splits;
   float lr, beta1, beta2, eps, bc1, bc2;
   int update;
   bf16 *W1b, *W2b, *W3b, *W2t, *W3t;

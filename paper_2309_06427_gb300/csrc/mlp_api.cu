@@ -68,8 +68,8 @@ bool qp_ok(const host::PlanView &v, const float *A, const float *B, const float 
   return true;
 }
 
-// Largest weight-gradient partial buffer: splits x max(W1 size, bias sizes).
-int64_t part_floats(int64_t rows) { return gemm_tn_splits(rows) * (int64_t)kHid * kIn; }
+// Gradients of every split, each laid out like the parameters.
+int64_t part_floats(int64_t rows) { return gemm_tn_splits(rows) * kParams; }
 
 sspcg_status refresh_copies(sspcg_mlp *n, cudaStream_t st) {
   AdamArgs a{};
@@ -94,17 +94,6 @@ sspcg_status forward(sspcg_mlp *n, const host::PlanView &v, int64_t row0, int64_
   MLP_CUDA(launch_gemm_nt(kEpiBiasRelu, n->X, n->W1b, rows, kHid, kIn, n->w + kB1, nullptr, n->H1, nullptr, st));
   MLP_CUDA(launch_gemm_nt(kEpiBiasRelu, n->H1, n->W2b, rows, kHid, kHid, n->w + kB2, nullptr, n->H2, nullptr, st));
   MLP_CUDA(launch_gemm_nt(kEpiBiasF32, n->H2, n->W3b, rows, kOut, kHid, n->w + kB3, nullptr, nullptr, n->Y, st));
-  return SSPCG_OK;
-}
-
-// Weight and bias gradients of one layer: dW[N1][N2] = G^T X, db = column sums of G.
-sspcg_status layer_grads(sspcg_mlp *n, const bf16 *G, int N1, const bf16 *Xin, int N2, int64_t rows, float *dW,
-                         float *db, cudaStream_t st) {
-  const int64_t splits = gemm_tn_splits(rows);
-  MLP_CUDA(launch_gemm_tn(G, N1, Xin, N2, rows, n->part, st));
-  MLP_CUDA(launch_reduce_splits(n->part, splits, (int64_t)N1 * N2, dW, st));
-  MLP_CUDA(launch_colsum(G, rows, N1, n->part, st));
-  MLP_CUDA(launch_reduce_splits(n->part, splits, N1, db, st));
   return SSPCG_OK;
 }
 
@@ -301,12 +290,15 @@ sspcg_status sspcg_mlp_train_step(sspcg_mlp *n, const sspcg_plan *plan, int32_t 
   la.Y = n->Y; la.lamstar = lambda_star; la.gamma = gamma; la.D = D; la.E = E;
   la.U = n->U; la.uu = n->uu; la.gg = n->gg; la.loss = loss; la.dY = n->dY;
   MLP_CUDA(launch_loss(la, st));
-  // backward: output layer, then the two hidden layers (ReLU masks from the stored activations)
-  if ((s = layer_grads(n, n->dY, kOut, n->H2, kHid, rows, n->g + kW3, n->g + kB3, st)) != SSPCG_OK) return s;
+  // backward: output layer, then the two hidden layers (ReLU masks from the stored activations); the splits of the
+  // gradients lie like the parameters
+  float *part = n->part;
+  MLP_CUDA(launch_gemm_tn(n->dY, kOut, n->H2, kHid, rows, part + kW3, st));
   MLP_CUDA(launch_gemm_nt(kEpiMask, n->dY, n->W3t, rows, kHid, kOut, nullptr, n->H2, n->dH2, nullptr, st));
-  if ((s = layer_grads(n, n->dH2, kHid, n->H1, kHid, rows, n->g + kW2, n->g + kB2, st)) != SSPCG_OK) return s;
+  MLP_CUDA(launch_gemm_tn(n->dH2, kHid, n->H1, kHid, rows, part + kW2, st));
   MLP_CUDA(launch_gemm_nt(kEpiMask, n->dH2, n->W2t, rows, kHid, kHid, nullptr, n->H1, n->dH1, nullptr, st));
-  if ((s = layer_grads(n, n->dH1, kHid, n->X, kIn, rows, n->g + kW1, n->g + kB1, st)) != SSPCG_OK) return s;
+  MLP_CUDA(launch_gemm_tn(n->dH1, kHid, n->X, kIn, rows, part + kW1, st));
+  MLP_CUDA(launch_colsum(n->dY, n->dH2, n->dH1, rows, part, st));
   // Adam
   n->t += 1;
   AdamArgs a{};
@@ -314,6 +306,8 @@ sspcg_status sspcg_mlp_train_step(sspcg_mlp *n, const sspcg_plan *plan, int32_t 
   a.lr = hyper->lr; a.beta1 = hyper->beta1; a.beta2 = hyper->beta2; a.eps = hyper->eps;
   a.bc1 = (float)(1.0 - std::pow((double)hyper->beta1, (double)n->t));
   a.bc2 = (float)(1.0 - std::pow((double)hyper->beta2, (double)n->t));
+  a.part = part;
+  a.splits = gemm_tn_splits(rows);
   a.update = 1;
   a.W1b = n->W1b; a.W2b = n->W2b; a.W3b = n->W3b; a.W2t = n->W2t; a.W3t = n->W3t;
   MLP_CUDA(launch_adam(a, st));
