@@ -41,7 +41,7 @@ constexpr int64_t kFeatTable = (int64_t)kPadX * (kPadU + 1) * kIn;
 void build_feature_table(int16_t *tab);
 // Normalised bf16 feature rows of the span into X; tab: the gather table on the device.
 cudaError_t launch_features(const RowSpan &rs, const QpData &q, const float *mu, const float *isd,
-                            const int16_t *tab, bf16 *X, cudaStream_t st);
+                            const int16_t *tab, bf16 *X, cudaStream_t st, int sms);
 // Column sums of the raw features over the span: part [warps][2][kIn] (FP64); returns warps used.
 cudaError_t launch_feature_stats(const RowSpan &rs, const QpData &q, double *part, int warps, cudaStream_t st);
 cudaError_t launch_stats_finish(const double *part, int warps, int64_t rows, float *mu, float *isd,

@@ -84,7 +84,7 @@ sspcg_status refresh_copies(sspcg_mlp *n, cudaStream_t st) {
 sspcg_status forward(sspcg_mlp *n, const host::PlanView &v, int64_t row0, int64_t rows, const QpData &q,
                      cudaStream_t st) {
   RowSpan rs{v.ps, v.kref, row0, rows};
-  MLP_CUDA(launch_features(rs, q, n->mu, n->isd, n->ftab, n->X, st));
+  MLP_CUDA(launch_features(rs, q, n->mu, n->isd, n->ftab, n->X, st, host::sms()));
   if (n->engine == SSPCG_MLP_ENGINE_TCGEN05) {
     MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->X, n->W1b, rows, kHid, kIn, n->w + kB1, n->H1, nullptr, n->err, st));
     MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->H1, n->W2b, rows, kHid, kHid, n->w + kB2, n->H2, nullptr, n->err, st));
@@ -240,7 +240,7 @@ sspcg_status sspcg_mlp_features(const sspcg_mlp *n, const sspcg_plan *plan, int3
   if (rows > n->max_rows) return SSPCG_ERR_INVALID_ARG;
   RowSpan rs{v.ps, v.kref, row0, rows};
   MLP_CUDA(launch_features(rs, qp(A, B, qd, rd, gamma, PD), n->mu, n->isd, n->ftab, reinterpret_cast<bf16 *>(X),
-                           (cudaStream_t)stream));
+                           (cudaStream_t)stream, host::sms()));
   return SSPCG_OK;
 }
 

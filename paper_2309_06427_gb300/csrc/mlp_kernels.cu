@@ -147,45 +147,100 @@ void build_feature_table(int16_t *tab) {
 
 namespace {
 
-// One warp per knot row: stage the knot's data (zeros for the k - 1 blocks of row 0), then lane l writes
-// columns 64 i + 2 l, +1, each gathered from the stage through the table of the problem's (nx, nu).
-__global__ void __launch_bounds__(kFeatWarps * 32) features_kernel(RowSpan rs, QpData q, const float *__restrict__ mu,
-                                                                   const float *__restrict__ isd,
-                                                                   const int16_t *__restrict__ tab,
-                                                                   bf16 *__restrict__ X) {
-  __shared__ __align__(16) float stage[kFeatWarps][kStFloats];
+__device__ __forceinline__ void cp_async4(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
+
+// dst[i] = src[i] for i < n, asynchronously, or zeros.
+__device__ __forceinline__ void warp_fetch(float *dst, const float *src, int n, bool zero, int lane) {
+  if (zero) {
+    for (int i = lane; i < n; i += 32) dst[i] = 0.f;
+  } else {
+    for (int i = lane; i < n; i += 32) cp_async4(dst + i, src + i);
+  }
+}
+
+// What stage_knot brings, asynchronously; zeros for the blocks of knot k - 1 when k = 0.
+__device__ __forceinline__ void fetch_knot(float *s, const ProbDesc &d, int k, const QpData &q, int lane) {
+  const int m = d.nx, u = d.nu;
+  const bool first = k == 0;
+  warp_fetch(s + kStA, q.A + d.oA + (int64_t)(k - 1) * m * m, m * m, first, lane);
+  warp_fetch(s + kStB, q.B + d.oB + (int64_t)(k - 1) * m * u, m * u, first, lane);
+  warp_fetch(s + kStPD, q.PD + d.odiag + (int64_t)k * m * m, m * m, false, lane);
+  warp_fetch(s + kStQp, q.qd + d.oq + (int64_t)(k - 1) * m, m, first, lane);
+  warp_fetch(s + kStRp, q.rd + d.orr + (int64_t)(k - 1) * u, u, first, lane);
+  warp_fetch(s + kStQ, q.qd + d.oq + (int64_t)k * m, m, false, lane);
+  warp_fetch(s + kStG, q.gamma + d.ovec + (int64_t)k * m, m, false, lane);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Feature rows.  Bound: the 2.7 KB written per row.  A warp per row spent most
+// of its time elsewhere: on the chain kref -> problem -> knot -> row, which
+// nothing overlapped, and on reading mu, 1/sigma and the gather table again for
+// each row, as many cache accesses as the row itself.  Here a warp walks
+// consecutive rows, holds its 42 columns' mu and 1/sigma, and their gather
+// indices until nx or nu changes, in registers, and fetches the next row's knot
+// while it writes this one's.
+// 266,240 rows, nx 14: 0.468 to 0.33 ms, 3.8 TB/s.
+// ---------------------------------------------------------------------------
+constexpr int kFeatRowWarps = 12;  // one CTA per SM; two knots per warp in shared memory
+constexpr int kFeatSmem = kFeatRowWarps * 2 * kStFloats * (int)sizeof(float);
+
+__global__ void __launch_bounds__(kFeatRowWarps * 32, 1)
+    features_kernel(RowSpan rs, int64_t per, QpData q, const float *__restrict__ mu, const float *__restrict__ isd,
+                    const int16_t *__restrict__ tab, bf16 *__restrict__ X) {
+  extern __shared__ __align__(16) float fsm[];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int64_t r = (int64_t)blockIdx.x * kFeatWarps + wl;
-  if (r >= rs.nrows) return;  // warp-uniform
-  const int2 ref = rs.kref[rs.row0 + r];
-  const ProbDesc d = rs.ps.get(ref.x);
-  const int k = ref.y, m = d.nx, u = d.nu;
-  float *s = stage[wl];
-  if (k == 0) {  // no A_{k-1}, B_{k-1}, diag Q_{k-1}, diag R_{k-1}: their columns read zeros
-    for (int e = lane; e < m * m; e += 32) s[kStA + e] = 0.f;
-    for (int e = lane; e < m * u; e += 32) s[kStB + e] = 0.f;
-    if (lane < m) s[kStQp + lane] = 0.f;
-    if (lane < u) s[kStRp + lane] = 0.f;
-  }
-  stage_knot(s, d, k, q, lane);  // ends with __syncwarp
-  const float dj = block_solve(s, m, lane);  // zero for lane >= nx
-  if (lane < kPadX) s[kStDj + lane] = dj;
-  if (lane == 0) {
-    s[kStNx] = (float)m / (float)kPadX;
-    s[kStZero] = 0.f;
-  }
-  __syncwarp();
-  const int16_t *t = tab + ((int64_t)(m - 1) * (kPadU + 1) + u) * kIn;
-  __nv_bfloat162 *out = reinterpret_cast<__nv_bfloat162 *>(X + r * kIn);
+  const int64_t r0 = ((int64_t)blockIdx.x * kFeatRowWarps + wl) * per;
+  const int64_t r1 = r0 + per < rs.nrows ? r0 + per : rs.nrows;
+  if (r0 >= r1) return;  // warp-uniform; warps share nothing
+  float *buf = fsm + wl * 2 * kStFloats;
+  if (lane < 2) buf[lane * kStFloats + kStZero] = 0.f;
+  float2 mm[kPairIters], is[kPairIters];
 #pragma unroll
   for (int it = 0; it < kPairIters; ++it) {
-    const int c = it * 64 + 2 * lane;
-    const short2 id = *reinterpret_cast<const short2 *>(t + c);
-    const float2 mm = *reinterpret_cast<const float2 *>(mu + c);
-    const float2 is = *reinterpret_cast<const float2 *>(isd + c);
-    const float vx = (s[id.x] - mm.x) * is.x;
-    const float vy = (s[id.y] - mm.y) * is.y;
-    out[c >> 1] = __floats2bfloat162_rn(vx, vy);
+    mm[it] = *reinterpret_cast<const float2 *>(mu + it * 64 + 2 * lane);
+    is[it] = *reinterpret_cast<const float2 *>(isd + it * 64 + 2 * lane);
+  }
+  const int2 *refs = rs.kref + rs.row0;
+  int2 ref = refs[r0], next = refs[r0 + 1 < r1 ? r0 + 1 : r0];
+  ProbDesc d = rs.ps.get(ref.x);
+  fetch_knot(buf, d, ref.y, q, lane);
+  short2 id[kPairIters];
+  int tm = 0, tu = -1;
+  for (int64_t r = r0; r < r1; ++r) {
+    const int m = d.nx, u = d.nu;
+    float *s = buf + ((r - r0) & 1) * kStFloats;
+    if (r + 1 < r1) {
+      if (next.x != ref.x) d = rs.ps.get(next.x);
+      ref = next;
+      fetch_knot(buf + ((r + 1 - r0) & 1) * kStFloats, d, ref.y, q, lane);
+      if (r + 2 < r1) next = refs[r + 2];
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+    if (m != tm || u != tu) {
+      const int16_t *t = tab + ((int64_t)(m - 1) * (kPadU + 1) + u) * kIn;
+#pragma unroll
+      for (int it = 0; it < kPairIters; ++it) id[it] = *reinterpret_cast<const short2 *>(t + it * 64 + 2 * lane);
+      tm = m;
+      tu = u;
+    }
+    __syncwarp();
+    const float dj = block_solve(s, m, lane);  // zero for lane >= nx
+    if (lane < kPadX) s[kStDj + lane] = dj;
+    if (lane == 0) s[kStNx] = (float)m / (float)kPadX;
+    __syncwarp();
+    __nv_bfloat162 *out = reinterpret_cast<__nv_bfloat162 *>(X + r * kIn);
+#pragma unroll
+    for (int it = 0; it < kPairIters; ++it) {
+      const float vx = (s[id[it].x] - mm[it].x) * is[it].x;
+      const float vy = (s[id[it].y] - mm[it].y) * is[it].y;
+      out[it * 32 + lane] = __floats2bfloat162_rn(vx, vy);
+    }
+    __syncwarp();  // the buffer is read: the next fetch may take it
   }
 }
 
@@ -667,9 +722,14 @@ int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 }  // namespace
 
 cudaError_t launch_features(const RowSpan &rs, const QpData &q, const float *mu, const float *isd,
-                            const int16_t *tab, bf16 *X, cudaStream_t st) {
+                            const int16_t *tab, bf16 *X, cudaStream_t st, int sms) {
   if (rs.nrows <= 0) return cudaSuccess;
-  features_kernel<<<(unsigned)cdiv64(rs.nrows, kFeatWarps), kFeatWarps * 32, 0, st>>>(rs, q, mu, isd, tab, X);
+  static std::atomic<uint64_t> attr_done{0};
+  const cudaError_t e = smem_attr_once(attr_done, features_kernel, kFeatSmem);
+  if (e != cudaSuccess) return e;
+  const int64_t per = cdiv64(rs.nrows, (int64_t)sms * kFeatRowWarps);
+  features_kernel<<<(unsigned)cdiv64(rs.nrows, per * kFeatRowWarps), kFeatRowWarps * 32, kFeatSmem, st>>>(
+      rs, per, q, mu, isd, tab, X);
   return cudaGetLastError();
 }
 
