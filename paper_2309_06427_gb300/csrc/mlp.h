@@ -55,7 +55,7 @@ cudaError_t launch_gemm_nt(int epi, const bf16 *A, const bf16 *B, int64_t M, int
 // The same product on the 5th-generation tensor cores (tcgen05 + TMA): N in {256, 32}, K % 64 == 0,
 // epilogues kEpiBiasRelu and kEpiBiasF32; *err is set to 1 when a bounded wait expires.
 cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, int N, int K, const float *bias,
-                              bf16 *Cb, float *Cf, int *err, cudaStream_t st);
+                              bf16 *Cb, float *Cf, int *err, cudaStream_t st, int sms);
 // False when the driver's tensor-map encoder is unavailable.
 bool tc_available();
 // part[s kParams + n1 N2 + n2] = sum over rows m of split s of G[m][n1] X[m][n2].

@@ -86,9 +86,13 @@ sspcg_status forward(sspcg_mlp *n, const host::PlanView &v, int64_t row0, int64_
   RowSpan rs{v.ps, v.kref, row0, rows};
   MLP_CUDA(launch_features(rs, q, n->mu, n->isd, n->ftab, n->X, st, host::sms()));
   if (n->engine == SSPCG_MLP_ENGINE_TCGEN05) {
-    MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->X, n->W1b, rows, kHid, kIn, n->w + kB1, n->H1, nullptr, n->err, st));
-    MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->H1, n->W2b, rows, kHid, kHid, n->w + kB2, n->H2, nullptr, n->err, st));
-    MLP_CUDA(launch_gemm_nt_tc(kEpiBiasF32, n->H2, n->W3b, rows, kOut, kHid, n->w + kB3, nullptr, n->Y, n->err, st));
+    const int sms = host::sms();
+    MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->X, n->W1b, rows, kHid, kIn, n->w + kB1, n->H1, nullptr, n->err, st,
+                               sms));
+    MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->H1, n->W2b, rows, kHid, kHid, n->w + kB2, n->H2, nullptr, n->err, st,
+                               sms));
+    MLP_CUDA(launch_gemm_nt_tc(kEpiBiasF32, n->H2, n->W3b, rows, kOut, kHid, n->w + kB3, nullptr, n->Y, n->err, st,
+                               sms));
     return SSPCG_OK;
   }
   MLP_CUDA(launch_gemm_nt(kEpiBiasRelu, n->X, n->W1b, rows, kHid, kIn, n->w + kB1, nullptr, n->H1, nullptr, st));

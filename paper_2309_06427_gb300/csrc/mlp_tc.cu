@@ -1,6 +1,6 @@
 // Warm-start network products on the 5th-generation tensor cores:
 // C[M][N] = epilogue(A[M][K] B[N][K]^T), bf16 operands, FP32 accumulation in
-// tensor memory.  One CTA (4 warps) per 128-row tile and the whole N (256 or
+// tensor memory.  One CTA (4 warps) per MT x 128 rows and the whole N (256 or
 // 32): warp 0 streams A and B tiles of 64 columns (128 bytes) into a ring of
 // shared-memory stages with TMA (128-byte swizzle); warp 1 issues
 // tcgen05.mma (M = 128, K = 16 per instruction) from one thread and
@@ -101,22 +101,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <int N>
+template <int N, int MT>
 struct TcCfg {
-  static constexpr int kStages = N >= 256 ? 4 : 6;
-  static constexpr int kABytes = kTcM * kTcK * 2;  // 16 KB
+  static constexpr int kStages = N >= 256 ? (MT == 2 ? 3 : 4) : 6;
+  static constexpr int kABytes = MT * kTcM * kTcK * 2;  // 16 KB per 128 rows
   static constexpr int kBBytes = N * kTcK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kTmemCols = N < 32 ? 32 : N;  // power of two >= 32
+  static constexpr int kTmemCols = MT * N;  // power of two >= 32
   static constexpr int kSmem = kStages * kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
 };
 
-template <int N, int EPI>
+template <int N, int EPI, int MT>
 __global__ void __launch_bounds__(kTcThreads, 1)
     gemm_nt_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int64_t M,
                       int K, const float *__restrict__ bias, bf16 *__restrict__ Cb, float *__restrict__ Cf,
                       int *__restrict__ err) {
-  using C = TcCfg<N>;
+  using C = TcCfg<N, MT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *stage_base = smem;
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __shared__ int failed;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t m0 = (int64_t)blockIdx.x * kTcM;
+  const int64_t m0 = (int64_t)blockIdx.x * kTcM * MT;
   const int KT = K / kTcK;
 
   if (threadIdx.x == 0) {
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    // producer: TMA loads of A rows [m0, m0 + 128) and all N rows of B, 64 columns per stage
+    // producer: TMA loads of A rows [m0, m0 + 128 MT) and all N rows of B, 64 columns per stage
     for (int kt = 0; kt < KT; ++kt) {
       const int s = kt % C::kStages;
       if (kt >= C::kStages && !mbar_wait(&empty[s], ((kt / C::kStages) - 1) & 1)) {
@@ -160,7 +160,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       uint8_t *a = stage_base + s * C::kStageBytes;
       uint8_t *b = a + C::kABytes;
       mbar_expect_tx(&full[s], C::kStageBytes);
-      tma_load_2d(a, &mapA, kt * kTcK, (int)m0, &full[s]);
+#pragma unroll
+      for (int t = 0; t < MT; ++t)
+        tma_load_2d(a + t * (C::kABytes / MT), &mapA, kt * kTcK, (int)m0 + t * kTcM, &full[s]);
       tma_load_2d(b, &mapB, kt * kTcK, 0, &full[s]);
     }
   } else if (warp == 1 && lane == 0) {
@@ -178,8 +180,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const uint8_t *a = stage_base + s * C::kStageBytes;
       const uint8_t *b = a + C::kABytes;
 #pragma unroll
-      for (int k = 0; k < kTcK / 16; ++k)
-        mma_issue(tmem, smem_desc(a + k * 32), smem_desc(b + k * 32), idesc, (kt > 0 || k > 0) ? 1u : 0u);
+      for (int t = 0; t < MT; ++t)
+#pragma unroll
+        for (int k = 0; k < kTcK / 16; ++k)
+          mma_issue(tmem + t * N, smem_desc(a + t * (C::kABytes / MT) + k * 32), smem_desc(b + k * 32), idesc,
+                    (kt > 0 || k > 0) ? 1u : 0u);
       mma_commit(&empty[s]);  // stage free once these products have read it
     }
     mma_commit(acc_full);  // accumulators complete
@@ -192,13 +197,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   __syncthreads();
   if (!failed) {
-    const int row_in_tile = warp * 32 + lane;
-    const int64_t row = m0 + row_in_tile;
     const uint32_t tbase = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
-    for (int c0 = 0; c0 < N; c0 += 16) {
+    for (int cc = 0; cc < MT * N; cc += 16) {
+      const int c0 = cc % N;
+      const int64_t row = m0 + cc / N * kTcM + warp * 32 + lane;
       float v[16];
-      tmem_ld16(tbase + (uint32_t)c0, v);
+      tmem_ld16(tbase + (uint32_t)cc, v);
       if (row < M) {
         if (EPI == kEpiBiasRelu) {
           uint32_t packed[8];
@@ -257,15 +262,15 @@ bool make_map(CUtensorMap *map, const bf16 *base, int64_t rows, int cols, int bo
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int N, int EPI>
+template <int N, int EPI, int MT>
 cudaError_t launch_tc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t M, int K, const float *bias, bf16 *Cb,
                       float *Cf, int *err, cudaStream_t st) {
-  using C = TcCfg<N>;
+  using C = TcCfg<N, MT>;
   static std::atomic<uint64_t> attr_done{0};
-  cudaError_t e = smem_attr_once(attr_done, gemm_nt_tc_kernel<N, EPI>, C::kSmem);
+  cudaError_t e = smem_attr_once(attr_done, gemm_nt_tc_kernel<N, EPI, MT>, C::kSmem);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((M + kTcM - 1) / kTcM);
-  gemm_nt_tc_kernel<N, EPI><<<grid, kTcThreads, C::kSmem, st>>>(ma, mb, M, K, bias, Cb, Cf, err);
+  const unsigned grid = (unsigned)((M + MT * kTcM - 1) / (MT * kTcM));
+  gemm_nt_tc_kernel<N, EPI, MT><<<grid, kTcThreads, C::kSmem, st>>>(ma, mb, M, K, bias, Cb, Cf, err);
   return cudaGetLastError();
 }
 
@@ -274,7 +279,7 @@ cudaError_t launch_tc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t M, i
 bool tc_available() { return encode_fn() != nullptr; }
 
 cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, int N, int K, const float *bias,
-                              bf16 *Cb, float *Cf, int *err, cudaStream_t st) {
+                              bf16 *Cb, float *Cf, int *err, cudaStream_t st, int sms) {
   if (M <= 0) return cudaSuccess;
   if (K % kTcK != 0 || K <= 0) return cudaErrorInvalidValue;
   if (!(N == 256 || N == 32)) return cudaErrorInvalidValue;
@@ -283,11 +288,16 @@ cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, 
   if ((reinterpret_cast<uintptr_t>(A) & 15u) || (reinterpret_cast<uintptr_t>(B) & 15u)) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
   if (!make_map(&ma, A, M, K, kTcM) || !make_map(&mb, B, N, K, N)) return cudaErrorInvalidValue;
+  // Two row tiles per CTA share each stage's B rows (256 KB instead of 384 KB of L2 reads per 128 rows and 256 columns,
+  // which is what bounds the first layer), once one tile per CTA no longer fits on the SMs in one wave.
+  const bool pair = M > (int64_t)kTcM * sms;
+  if (N == 256 && epi == kEpiBiasRelu && pair)
+    return launch_tc<256, kEpiBiasRelu, 2>(ma, mb, M, K, bias, Cb, Cf, err, st);
   if (N == 256)
-    return epi == kEpiBiasRelu ? launch_tc<256, kEpiBiasRelu>(ma, mb, M, K, bias, Cb, Cf, err, st)
-                               : launch_tc<256, kEpiBiasF32>(ma, mb, M, K, bias, Cb, Cf, err, st);
-  return epi == kEpiBiasRelu ? launch_tc<32, kEpiBiasRelu>(ma, mb, M, K, bias, Cb, Cf, err, st)
-                             : launch_tc<32, kEpiBiasF32>(ma, mb, M, K, bias, Cb, Cf, err, st);
+    return epi == kEpiBiasRelu ? launch_tc<256, kEpiBiasRelu, 1>(ma, mb, M, K, bias, Cb, Cf, err, st)
+                               : launch_tc<256, kEpiBiasF32, 1>(ma, mb, M, K, bias, Cb, Cf, err, st);
+  return epi == kEpiBiasRelu ? launch_tc<32, kEpiBiasRelu, 1>(ma, mb, M, K, bias, Cb, Cf, err, st)
+                             : launch_tc<32, kEpiBiasF32, 1>(ma, mb, M, K, bias, Cb, Cf, err, st);
 }
 
 }  // namespace mlp
