@@ -114,6 +114,26 @@ __device__ __forceinline__ T warp_sum_split(T a, T b) {
   return half_warp_sum(red_add(keep, red_shfl_xor(give, 16)));
 }
 
+// Sum of nw <= 16 slots in every lane of a half-warp (l16: lane in the half).
+template <typename T>
+__device__ __forceinline__ T slot_sum(const T *slots, int l16, int nw, T zero) {
+  return half_warp_sum(l16 < nw ? slots[l16] : zero);
+}
+// In FP64 a butterfly over the next power of two of slots, repeated across the half: the steps that would only add
+// zeros change no bit, and an FP64 addition keeps its SM quarter's unit for 76 cycles whatever it adds (eight of them
+// per iteration and warp in CTAs of one warp; 16,384 problems, N 8-32, nx 2, 4, 6: 11.36 to 10.92 ms; nx 2, N 20 alone:
+// 102 to 96 us).  Double-float additions are cheap next to the branches: there the full butterfly stays.
+__device__ __forceinline__ double slot_sum(const double *slots, int l16, int nw, double zero) {
+  const int span = nw > 8 ? 16 : nw > 4 ? 8 : nw > 2 ? 4 : nw;
+  const int l = l16 & (span - 1);
+  double v = l < nw ? slots[l] : zero;
+  if (span > 8) v = red_add(v, red_shfl_xor(v, 8));
+  if (span > 4) v = red_add(v, red_shfl_xor(v, 4));
+  if (span > 2) v = red_add(v, red_shfl_xor(v, 2));
+  if (span > 1) v = red_add(v, red_shfl_xor(v, 1));
+  return v;
+}
+
 // Block-wide sum of K accumulators, every thread holding bit-identical results: warp sums, one slot per warp,
 // one barrier, then every warp sums the slots (at most 16: CTAs have at most 512 threads) in the same order.
 // Pairs of accumulators go through warp_sum_split, a single one through a full butterfly; the second stage
@@ -137,11 +157,11 @@ __device__ __forceinline__ void block_sum(typename R::T (&v)[K], typename R::T *
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < P; ++q) {
-    const T w = half_warp_sum(l16 < nw ? slots[(2 * q + h) * 32 + l16] : R::zero());
+    const T w = slot_sum(slots + (2 * q + h) * 32, l16, nw, R::zero());
     v[2 * q] = red_shfl(w, 0);
     v[2 * q + 1] = red_shfl(w, 16);
   }
-  if constexpr (K % 2 == 1) v[K - 1] = half_warp_sum(l16 < nw ? slots[(K - 1) * 32 + l16] : R::zero());
+  if constexpr (K % 2 == 1) v[K - 1] = slot_sum(slots + (K - 1) * 32, l16, nw, R::zero());
 }
 
 // The thread group that solves one problem: the CTA, or one warp (WARP: several problems per CTA, one per
