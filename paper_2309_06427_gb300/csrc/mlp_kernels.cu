@@ -587,14 +587,16 @@ __global__ void __launch_bounds__(kColThreads) colsum_kernel(const bf16 *__restr
 // (S_{k,k-1} = E_{k-1} in the packed [N][nx][nx] layout, S_{k,k+1} = its
 // transpose); then dL/dlambda0 = 2 S u / (P ||gamma||^2).
 // ---------------------------------------------------------------------------
-constexpr int kLossThreads = 256;
+constexpr int kLossThreads = 1024;  // a row per thread for most problems: a row is one chain of loads
 
+// Sum over the CTA, for warp 0 (FP64 additions are too dear for every warp to repeat them).
 __device__ __forceinline__ double block_sum_d(double v, double *slots) {
   v = warp_sum(v);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __syncthreads();
   if (lane == 0) slots[w] = v;
   __syncthreads();
+  if (w > 0) return 0.0;
   double s = 0.0;
   for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += slots[i];
   return s;
