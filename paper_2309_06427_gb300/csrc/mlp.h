@@ -56,6 +56,9 @@ cudaError_t launch_gemm_nt(int epi, const bf16 *A, const bf16 *B, int64_t M, int
 // epilogues kEpiBiasRelu and kEpiBiasF32; *err is set to 1 when a bounded wait expires.
 cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, int N, int K, const float *bias,
                               bf16 *Cb, float *Cf, int *err, cudaStream_t st, int sms);
+// lambda rows of the span from H1 [nrows][kHid]: the second and third layer and the scatter (tcgen05 engine).
+cudaError_t launch_tail_tc(const RowSpan &rs, const bf16 *H1, const bf16 *W2, const float *b2, const bf16 *W3,
+                           const float *b3, float *lambda, int *err, cudaStream_t st, int sms);
 // False when the driver's tensor-map encoder is unavailable.
 bool tc_available();
 // part[s kParams + n1 N2 + n2] = sum over rows m of split s of G[m][n1] X[m][n2].

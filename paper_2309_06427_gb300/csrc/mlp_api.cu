@@ -260,9 +260,18 @@ sspcg_status sspcg_mlp_infer(sspcg_mlp *n, const sspcg_plan *plan, const float *
   const QpData q = qp(A, B, qd, rd, gamma, PD);
   for (int64_t r0 = 0; r0 < v.knots; r0 += n->max_rows) {
     const int64_t rows = std::min<int64_t>(n->max_rows, v.knots - r0);
+    const RowSpan rs{v.ps, v.kref, r0, rows};
+    if (n->engine == SSPCG_MLP_ENGINE_TCGEN05) {
+      const int sms = host::sms();
+      MLP_CUDA(launch_features(rs, q, n->mu, n->isd, n->ftab, n->X, st, sms));
+      MLP_CUDA(launch_gemm_nt_tc(kEpiBiasRelu, n->X, n->W1b, rows, kHid, kIn, n->w + kB1, n->H1, nullptr, n->err, st,
+                                 sms));
+      MLP_CUDA(launch_tail_tc(rs, n->H1, n->W2b, n->w + kB2, n->W3b, n->w + kB3, lambda0, n->err, st, sms));
+      continue;
+    }
     sspcg_status s = forward(n, v, r0, rows, q, st);
     if (s != SSPCG_OK) return s;
-    MLP_CUDA(launch_scatter_lambda(RowSpan{v.ps, v.kref, r0, rows}, n->Y, lambda0, st));
+    MLP_CUDA(launch_scatter_lambda(rs, n->Y, lambda0, st));
   }
   return SSPCG_OK;
 }

@@ -236,6 +236,157 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if (threadIdx.x == 0 && failed) atomicExch(err, 1);
 }
 
+// ---------------------------------------------------------------------------
+// Inference after its first layer, in one kernel:
+//   lambda0 = rows of (relu(H1 W2^T + b2) W3^T + b3), H1 [M][256] of a span.
+// As separate products and a scatter these were three launches that write and
+// read H2 (0.5 KB per row each way) and Y, and the 256-column one spent its time
+// between tiles: four stages of K, then an epilogue that nothing overlapped.
+// Here a CTA per SM keeps both weight matrices (144 KB) in shared memory and
+// walks the row tiles: TMA brings 128 rows of H1, the epilogue of the second
+// layer writes H2 over them as the third layer's operand (128-byte swizzle: the
+// 16-byte piece p of row r lies at piece p ^ (r % 8)), and the third layer's
+// epilogue writes lambda0.  The next tile's H1 is on its way meanwhile.  The
+// products and roundings are those of gemm_nt_tc_kernel in the same order, so
+// lambda0 is bit-identical.  266,240 rows: 208 us in three launches before,
+// 82 us now, bound by the serial chain of a tile: load, two products, two epilogues.
+// ---------------------------------------------------------------------------
+constexpr int kTailThreads = 256;  // eight warps: two per quarter of the TMEM lanes
+constexpr int kTailKT = kHid / kTcK;
+// bytes per 64 columns
+constexpr int kTailABytes = kTcM * kTcK * 2, kTailW2Bytes = kHid * kTcK * 2, kTailW3Bytes = kOut * kTcK * 2;
+constexpr int kTailSmem = kTailKT * (kTailABytes + kTailW2Bytes + kTailW3Bytes) + 1024 /*alignment*/;
+
+__global__ void __launch_bounds__(kTailThreads, 1)
+    tail_tc_kernel(const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapW2,
+                   const __grid_constant__ CUtensorMap mapW3, RowSpan rs, const float *__restrict__ b2,
+                   const float *__restrict__ b3, float *__restrict__ lambda, int *__restrict__ err) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *sW2 = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *sA = sW2 + kTailKT * kTailW2Bytes, *sW3 = sA + kTailKT * kTailABytes;
+  __shared__ uint64_t bar_w, bar_a, bar_2, bar_3;  // weights and H1 arrived; second and third layer done
+  __shared__ uint32_t tmem_slot;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t tiles = (rs.nrows + kTcM - 1) / kTcM;
+  const bool first = threadIdx.x == 0;
+  auto load_tile = [&](int64_t tile) {
+    mbar_expect_tx(&bar_a, kTailKT * kTailABytes);
+    for (int kt = 0; kt < kTailKT; ++kt)
+      tma_load_2d(sA + kt * kTailABytes, &mapH, kt * kTcK, (int)(tile * kTcM), &bar_a);
+  };
+
+  if (first) {
+    mbar_init(&bar_w, 1);
+    mbar_init(&bar_a, 1);
+    mbar_init(&bar_2, 1);
+    mbar_init(&bar_3, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    mbar_expect_tx(&bar_w, kTailKT * (kTailW2Bytes + kTailW3Bytes));
+    for (int kt = 0; kt < kTailKT; ++kt) {
+      tma_load_2d(sW2 + kt * kTailW2Bytes, &mapW2, kt * kTcK, 0, &bar_w);
+      tma_load_2d(sW3 + kt * kTailW3Bytes, &mapW3, kt * kTcK, 0, &bar_w);
+    }
+    load_tile(blockIdx.x);  // the grid is at most the tiles
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(su32(&tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  const uint32_t tmem = tmem_slot, acc3 = tmem + kHid;  // accumulators: columns 0-255 and 256-287
+  const int quarter = warp & 3, r = quarter * 32 + lane;
+  const uint32_t tlane = (uint32_t)(quarter * 32) << 16;
+  bool ok = true;
+  uint32_t parity = 0;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, parity ^= 1) {
+    if (first) {
+      ok = mbar_wait(&bar_w, 0) && mbar_wait(&bar_a, parity);
+      if (ok) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        for (int kt = 0; kt < kTailKT; ++kt)
+#pragma unroll
+          for (int k = 0; k < kTcK / 16; ++k)
+            mma_issue(tmem, smem_desc(sA + kt * kTailABytes + k * 32), smem_desc(sW2 + kt * kTailW2Bytes + k * 32),
+                      instr_desc(kTcM, kHid), (kt > 0 || k > 0) ? 1u : 0u);
+        mma_commit(&bar_2);
+      }
+    }
+    __syncwarp();
+    ok = mbar_wait(&bar_2, parity) && ok;
+    ok = __all_sync(0xffffffffu, ok);
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (ok) {
+      // H2 over H1, which the second layer has read
+#pragma unroll 1
+      for (int c0 = (warp >> 2) * (kHid / 2); c0 < ((warp >> 2) + 1) * (kHid / 2); c0 += 16) {
+        float v[16];
+        tmem_ld16(tmem + tlane + (uint32_t)c0, v);
+        uint32_t packed[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(v[2 * i] + __ldg(b2 + c0 + 2 * i), 0.f),
+                                                         fmaxf(v[2 * i + 1] + __ldg(b2 + c0 + 2 * i + 1), 0.f));
+          packed[i] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        uint8_t *row = sA + (c0 / kTcK) * kTailABytes + r * 128;
+        const int piece = (c0 % kTcK) / 8;
+        *reinterpret_cast<uint4 *>(row + ((piece ^ (r & 7)) << 4)) =
+            make_uint4(packed[0], packed[1], packed[2], packed[3]);
+        *reinterpret_cast<uint4 *>(row + (((piece + 1) ^ (r & 7)) << 4)) =
+            make_uint4(packed[4], packed[5], packed[6], packed[7]);
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      break;
+    }
+    if (first) {
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      for (int kt = 0; kt < kTailKT; ++kt)
+#pragma unroll
+        for (int k = 0; k < kTcK / 16; ++k)
+          mma_issue(acc3, smem_desc(sA + kt * kTailABytes + k * 32), smem_desc(sW3 + kt * kTailW3Bytes + k * 32),
+                    instr_desc(kTcM, kOut), (kt > 0 || k > 0) ? 1u : 0u);
+      mma_commit(&bar_3);
+    }
+    __syncwarp();
+    ok = __all_sync(0xffffffffu, mbar_wait(&bar_3, parity));
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      break;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (first && tile + gridDim.x < tiles) load_tile(tile + gridDim.x);  // the third layer has read H2
+    __syncwarp();
+    if (warp < 4) {
+      float v[32];
+      tmem_ld16(acc3 + tlane, *reinterpret_cast<float(*)[16]>(v));
+      tmem_ld16(acc3 + tlane + 16, *reinterpret_cast<float(*)[16]>(v + 16));
+      const int64_t row = tile * kTcM + r;
+      if (row < rs.nrows) {
+        const int2 ref = rs.kref[rs.row0 + row];
+        const ProbDesc d = rs.ps.get(ref.x);
+        float *o = lambda + d.ovec + (int64_t)ref.y * d.nx;
+#pragma unroll
+        for (int i = 0; i < kPadX; ++i)
+          if (i < d.nx) o[i] = v[i] + __ldg(b3 + i);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  if (warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512));
+  }
+  if (first && !ok) atomicExch(err, 1);
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -298,6 +449,22 @@ cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, 
                                : launch_tc<256, kEpiBiasF32, 1>(ma, mb, M, K, bias, Cb, Cf, err, st);
   return epi == kEpiBiasRelu ? launch_tc<32, kEpiBiasRelu, 1>(ma, mb, M, K, bias, Cb, Cf, err, st)
                              : launch_tc<32, kEpiBiasF32, 1>(ma, mb, M, K, bias, Cb, Cf, err, st);
+}
+
+cudaError_t launch_tail_tc(const RowSpan &rs, const bf16 *H1, const bf16 *W2, const float *b2, const bf16 *W3,
+                           const float *b3, float *lambda, int *err, cudaStream_t st, int sms) {
+  if (rs.nrows <= 0) return cudaSuccess;
+  CUtensorMap mh, m2, m3;
+  if (!make_map(&mh, H1, rs.nrows, kHid, kTcM) || !make_map(&m2, W2, kHid, kHid, kHid) ||
+      !make_map(&m3, W3, kOut, kHid, kOut))
+    return cudaErrorInvalidValue;
+  static std::atomic<uint64_t> attr_done{0};
+  cudaError_t e = smem_attr_once(attr_done, tail_tc_kernel, kTailSmem);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (rs.nrows + kTcM - 1) / kTcM;
+  tail_tc_kernel<<<(unsigned)(tiles < sms ? tiles : sms), kTailThreads, kTailSmem, st>>>(mh, m2, m3, rs, b2, b3, lambda,
+                                                                                         err);
+  return cudaGetLastError();
 }
 
 }  // namespace mlp
