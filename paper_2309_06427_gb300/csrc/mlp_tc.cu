@@ -1,7 +1,7 @@
 // Warm-start network products on the 5th-generation tensor cores:
 // C[M][N] = epilogue(A[M][K] B[N][K]^T), bf16 operands, FP32 accumulation in
-// tensor memory.  One CTA (4 warps) per MT x 128 rows and the whole N (256 or
-// 32): warp 0 streams A and B tiles of 64 columns (128 bytes) into a ring of
+// tensor memory.  One CTA (4 warps) per MT x 128 rows and N (256, 64 or 32)
+// columns of C: warp 0 streams A and B tiles of 64 columns (128 bytes) into a ring of
 // shared-memory stages with TMA (128-byte swizzle); warp 1 issues
 // tcgen05.mma (M = 128, K = 16 per instruction) from one thread and
 // releases each stage with tcgen05.commit; then all four warps read the
@@ -103,7 +103,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 
 template <int N, int MT>
 struct TcCfg {
-  static constexpr int kStages = N >= 256 ? (MT == 2 ? 3 : 4) : 6;
+  static constexpr int kStages = N >= 256 ? (MT == 2 ? 3 : 4) : N == 64 ? 8 : 6;
   static constexpr int kABytes = MT * kTcM * kTcK * 2;  // 16 KB per 128 rows
   static constexpr int kBBytes = N * kTcK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
@@ -114,7 +114,7 @@ struct TcCfg {
 template <int N, int EPI, int MT>
 __global__ void __launch_bounds__(kTcThreads, 1)
     gemm_nt_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int64_t M,
-                      int K, const float *__restrict__ bias, bf16 *__restrict__ Cb, float *__restrict__ Cf,
+                      int K, int ldc, const float *__restrict__ bias, bf16 *__restrict__ Cb, float *__restrict__ Cf,
                       int *__restrict__ err) {
   using C = TcCfg<N, MT>;
   extern __shared__ uint8_t smem_raw[];
@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t m0 = (int64_t)blockIdx.x * kTcM * MT;
+  const int n0 = blockIdx.y * N;  // first column of C
   const int KT = K / kTcK;
 
   if (threadIdx.x == 0) {
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    // producer: TMA loads of A rows [m0, m0 + 128 MT) and all N rows of B, 64 columns per stage
+    // producer: TMA loads of A rows [m0, m0 + 128 MT) and B rows [n0, n0 + N), 64 columns per stage
     for (int kt = 0; kt < KT; ++kt) {
       const int s = kt % C::kStages;
       if (kt >= C::kStages && !mbar_wait(&empty[s], ((kt / C::kStages) - 1) & 1)) {
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
       for (int t = 0; t < MT; ++t)
         tma_load_2d(a + t * (C::kABytes / MT), &mapA, kt * kTcK, (int)m0 + t * kTcM, &full[s]);
-      tma_load_2d(b, &mapB, kt * kTcK, 0, &full[s]);
+      tma_load_2d(b, &mapB, kt * kTcK, n0, &full[s]);
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t tbase = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
     for (int cc = 0; cc < MT * N; cc += 16) {
-      const int c0 = cc % N;
+      const int c0 = n0 + cc % N;
       const int64_t row = m0 + cc / N * kTcM + warp * 32 + lane;
       float v[16];
       tmem_ld16(tbase + (uint32_t)cc, v);
@@ -214,11 +215,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
             packed[i] = *reinterpret_cast<const uint32_t *>(&h);
           }
-          uint4 *dst = reinterpret_cast<uint4 *>(Cb + row * N + c0);
+          uint4 *dst = reinterpret_cast<uint4 *>(Cb + row * ldc + c0);
           dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
           dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
         } else {
-          float4 *dst = reinterpret_cast<float4 *>(Cf + row * N + c0);
+          float4 *dst = reinterpret_cast<float4 *>(Cf + row * ldc + c0);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
             dst[i] = make_float4(v[4 * i] + bias[c0 + 4 * i], v[4 * i + 1] + bias[c0 + 4 * i + 1],
@@ -414,14 +415,14 @@ bool make_map(CUtensorMap *map, const bf16 *base, int64_t rows, int cols, int bo
 }
 
 template <int N, int EPI, int MT>
-cudaError_t launch_tc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t M, int K, const float *bias, bf16 *Cb,
-                      float *Cf, int *err, cudaStream_t st) {
+cudaError_t launch_tc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t M, int ldc, int K, const float *bias,
+                      bf16 *Cb, float *Cf, int *err, cudaStream_t st) {
   using C = TcCfg<N, MT>;
   static std::atomic<uint64_t> attr_done{0};
   cudaError_t e = smem_attr_once(attr_done, gemm_nt_tc_kernel<N, EPI, MT>, C::kSmem);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((M + MT * kTcM - 1) / (MT * kTcM));
-  gemm_nt_tc_kernel<N, EPI, MT><<<grid, kTcThreads, C::kSmem, st>>>(ma, mb, M, K, bias, Cb, Cf, err);
+  const dim3 grid((unsigned)((M + MT * kTcM - 1) / (MT * kTcM)), (unsigned)(ldc / N));
+  gemm_nt_tc_kernel<N, EPI, MT><<<grid, kTcThreads, C::kSmem, st>>>(ma, mb, M, K, ldc, bias, Cb, Cf, err);
   return cudaGetLastError();
 }
 
@@ -437,18 +438,24 @@ cudaError_t launch_gemm_nt_tc(int epi, const bf16 *A, const bf16 *B, int64_t M, 
   if (!(epi == kEpiBiasRelu || epi == kEpiBiasF32)) return cudaErrorInvalidValue;
   // TMA needs 16-byte aligned bases and row strides (K * 2 bytes: K % 64 == 0)
   if ((reinterpret_cast<uintptr_t>(A) & 15u) || (reinterpret_cast<uintptr_t>(B) & 15u)) return cudaErrorInvalidValue;
+  // Few row tiles: each stage of a 256-column CTA is 48 KB, which one SM takes in at its own rate however idle the
+  // others are, so four CTAs share a row tile's columns as long as all of them run at once.  2,080 rows: the
+  // training step 156.8 to 144.6 us.
+  const int64_t tiles = (M + kTcM - 1) / kTcM;
+  const bool quarter = N == 256 && epi == kEpiBiasRelu && 4 * tiles <= sms;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A, M, K, kTcM) || !make_map(&mb, B, N, K, N)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, A, M, K, kTcM) || !make_map(&mb, B, N, K, quarter ? 64 : N)) return cudaErrorInvalidValue;
+  if (quarter) return launch_tc<64, kEpiBiasRelu, 1>(ma, mb, M, N, K, bias, Cb, Cf, err, st);
   // Two row tiles per CTA share each stage's B rows (256 KB instead of 384 KB of L2 reads per 128 rows and 256 columns,
   // which is what bounds the first layer), once one tile per CTA no longer fits on the SMs in one wave.
   const bool pair = M > (int64_t)kTcM * sms;
   if (N == 256 && epi == kEpiBiasRelu && pair)
-    return launch_tc<256, kEpiBiasRelu, 2>(ma, mb, M, K, bias, Cb, Cf, err, st);
+    return launch_tc<256, kEpiBiasRelu, 2>(ma, mb, M, N, K, bias, Cb, Cf, err, st);
   if (N == 256)
-    return epi == kEpiBiasRelu ? launch_tc<256, kEpiBiasRelu, 1>(ma, mb, M, K, bias, Cb, Cf, err, st)
-                               : launch_tc<256, kEpiBiasF32, 1>(ma, mb, M, K, bias, Cb, Cf, err, st);
-  return epi == kEpiBiasRelu ? launch_tc<32, kEpiBiasRelu, 1>(ma, mb, M, K, bias, Cb, Cf, err, st)
-                             : launch_tc<32, kEpiBiasF32, 1>(ma, mb, M, K, bias, Cb, Cf, err, st);
+    return epi == kEpiBiasRelu ? launch_tc<256, kEpiBiasRelu, 1>(ma, mb, M, N, K, bias, Cb, Cf, err, st)
+                               : launch_tc<256, kEpiBiasF32, 1>(ma, mb, M, N, K, bias, Cb, Cf, err, st);
+  return epi == kEpiBiasRelu ? launch_tc<32, kEpiBiasRelu, 1>(ma, mb, M, N, K, bias, Cb, Cf, err, st)
+                             : launch_tc<32, kEpiBiasF32, 1>(ma, mb, M, N, K, bias, Cb, Cf, err, st);
 }
 
 cudaError_t launch_tail_tc(const RowSpan &rs, const bf16 *H1, const bf16 *W2, const float *b2, const bf16 *W3,

@@ -51,6 +51,11 @@ def test_small_tiles(max_rows):
     _check(SHAPES[3:6] if max_rows == 1 else SHAPES, max_rows)
 
 
+@pytest.mark.parametrize("rows", [WAVE // 4, WAVE // 4 + 1])  # four CTAs per row tile, and the first size with one
+def test_around_a_quarter_wave(rows):
+    _check([(1023, 3, 2)] * (rows // 1024) + [(rows % 1024 - 1, 3, 2)], rows)
+
+
 @pytest.mark.parametrize("rows", [WAVE, WAVE + 1, WAVE + 128, WAVE + 129, 2 * WAVE + 256])
 def test_around_a_wave(rows):
     _check([(1023, 3, 2)] * (rows // 1024) + [(rows % 1024 - 1, 3, 2)] * (rows % 1024 > 0), rows)
