@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kSchurThreads) schur_f32_kernel(ProbSet ps, in
   const int tid = threadIdx.x;
   const ProbDesc d = ps.get(blockIdx.x / per);
   const int N = d.N, nx = d.nx, nu = d.nu, nn = nx * nx, m = nx + nu, nt = tiles4(nx), ld = 4 * nt;
-  const int ntl = nt * (nt + 1) / 2, C = schur_chunk(nx, nu);
+  const int ntl = nt * (nt + 1) / 2, C = chunk_share(schur_chunk(nx, nu), N, per);
   const Divisor by_nx(nx), by_nu(nu), by_ntl(ntl);
   const int part = blockIdx.x % per;
   if (part == 0) {
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kOffThreads, 4) precond_off_f32_kernel(ProbSet
   const int tid = threadIdx.x;
   const ProbDesc d = ps.get(blockIdx.x / per);
   const int N = d.N, nx = d.nx, nn = nx * nx, nt = tiles4(nx), ld = 4 * nt, blk = nx * ld, ntl = nt * nt;
-  const int C = off_chunk(nx);
+  const int C = chunk_share(off_chunk(nx), N, per);
   const Divisor by_ntl(ntl), by_nt(nt);
   for (int b0 = (int)(blockIdx.x % per) * C; b0 < N; b0 += per * C) {
     const int nb = min(C, N - b0);

@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(kKktThreads)
   __shared__ float sg[kChunkItems + kMaxNx];  // scaled gradients q_k / qd_k, r_k / rd_k, nx + nu per block
   const int tid = threadIdx.x;
   const ProbDesc d = ps.get(blockIdx.x / per);
-  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu, C = chunk_rows(nx, nu);
+  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu,
+            C = chunk_share(chunk_rows(nx, nu), N + 1, per);
   const int lda = nx | 1, ldb = nu | 1;
   const Divisor by_m(m), by_nx(nx);
   float *sA = sm, *sB = sm + C * nx * lda;
@@ -75,7 +76,8 @@ __global__ void __launch_bounds__(kKktThreads)
   __shared__ float sm[kChunkItems + kMaxNx];  // mu_{k+1} of the chunk's block rows
   const int tid = threadIdx.x;
   const ProbDesc d = ps.get(blockIdx.x / per);
-  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu, C = chunk_rows(nx, nu);
+  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu,
+            C = chunk_share(chunk_rows(nx, nu), N + 1, per);
   const Divisor by_m(m);
   for (int k0 = (int)(blockIdx.x % per) * C; k0 <= N; k0 += per * C) {
     const int k1 = min(N + 1, k0 + C), nb = min(k1, N) - k0;

@@ -24,7 +24,7 @@ SHAPES = [(N, nx, nu) for c, nx, nu in [(3, 28, 28), (6, 28, 0), (19, 5, 28), (2
 
 @pytest.mark.parametrize("kind", ["sym", "add", "bj", "jacobi"])
 def test_blocks_at_tile_and_chunk_ends(kind):
-    probs = P.custom_problems(SHAPES, config=84)
+    probs = P.custom_problems(SHAPES, config=84) * 170  # 6,120 problems: one CTA each, in full chunks
     plan = sspcg.sspcg_plan_create([p.N for p in probs], [p.nx for p in probs], [p.nu for p in probs], sspcg.options())
     b = sspcg.Batch(plan, probs)
     d = b.dev
@@ -34,7 +34,11 @@ def test_blocks_at_tile_and_chunk_ends(kind):
     diag, off = [(p.n, p.nx, p.nx) for p in probs], [(p.N, p.nx, p.nx) for p in probs]
     Ds, PDs = plan.unpack(sspcg.ARRAY_DIAG, b.D, diag), plan.unpack(sspcg.ARRAY_DIAG, b.PD, diag)
     Es, PEs = plan.unpack(sspcg.ARRAY_OFF, b.E, off), plan.unpack(sspcg.ARRAY_OFF, b.PE, off)
-    for i, p in enumerate(probs):
+    for i in range(len(SHAPES), len(probs)):
+        j = i % len(SHAPES)
+        for x in (Ds, Es, PDs, PEs):
+            assert np.array_equal(x[i], x[j]), SHAPES[j]
+    for i, p in enumerate(probs[:len(SHAPES)]):
         nd, no = p.n * p.nx ** 2, p.N * p.nx ** 2
         _, D, E = gpu_schur(p)
         assert np.array_equal(Ds[i].ravel(), D.cpu().numpy()[:nd]), SHAPES[i]
