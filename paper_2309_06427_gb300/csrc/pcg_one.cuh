@@ -1,8 +1,10 @@
 // PCG with a thread per row pair: the FP32 kernel for problems that fit in
 // shared memory whole and have at most one row pair per thread (textbook PCG,
 // double-float sums, degree-0 preconditioner; both operator forms).  The
-// iteration is the one of pcg.cuh, product for product and in the same order
-// of sums; what differs is where the values live.
+// iteration is the one of pcg.cuh and every block product is formed in the same
+// order; what differs is where the values live, and that the block sums group
+// rows 2c and 2c + 1 of a thread where pcg.cuh groups rows t, t + T, ..., so that
+// alpha and beta agree to a rounding of the double-float sum to FP32.
 //
 // pcg.cuh gives a thread single rows, takes one 32-bit shared-memory load per
 // multiply-add and keeps every vector in shared memory.  With one problem of
@@ -17,51 +19,22 @@
 //     multiply-add where a tile holds them side by side (products by rows);
 //   - the pair's entries of r, p, w, z, x and 1/q stay in registers; only r, p
 //     and v pass through shared memory, and x and w have no vector there, so
-//     that more problems fit whole (nx = 14: N <= 72 instead of 67);
-//   - the double-float sums fold their low part back only at the end (LazyDf),
-//     so that a step of a butterfly is one addition deep.
+//     that more problems fit whole (nx = 14, nu = 7: N <= 71 instead of 68).
 // Measured (GB300; us per iteration with one problem on each SM, pcg.cuh
-// before): nx = 14, N = 64: 5.02 -> 3.62; nx = 21, N = 30: 5.30 -> 3.70; nx = 4,
-// N = 64: 2.34 -> 1.28, and 1520 of them at once 618 -> 360 us in all.  Results
-// are bit-identical.
-// What bounds it: the shared-memory load pipe for the larger blocks (6,000 of
-// 7,000 cycles at nx = 14: every matrix entry comes through it once per use, a
-// third of the tile loads by columns with two-way bank conflicts where a warp
-// phase crosses a block row), the latency of five barriers and two block sums
-// for the smaller ones (2,400 cycles at nx = 4).
+// before): nx = 14, N = 64: 4.74 -> 3.52; nx = 21, N = 30: 5.01 -> 3.56; nx = 4,
+// N = 64: 2.20 -> 1.42, and 1520 of them at once 6.97 -> 4.41.  The sums are
+// pcg.cuh's, renormalised after every addition: folding the low parts only at
+// the end takes 5 % (nx = 14) to 15 % (nx = 4) less and leaves the sums 1.2
+// times (terms of one sign) to 1.9 times as far from the exact ones.
+// What bounds it: the shared-memory load pipe for the larger blocks (every
+// matrix entry comes through it once per use, a third of the tile loads by
+// columns with two-way bank conflicts where a warp phase crosses a block row),
+// the latency of five barriers and two block sums for the smaller ones.
 #pragma once
 
 #include "pcg.cuh"
 
 namespace sspcg {
-
-// Double-float accumulator of this kernel: the products are exact, the high parts are summed with TwoSum and every
-// error goes to the low part, which get() folds in at the end.  A block sum adds few enough terms (two products and
-// at most nine partial sums deep) that the low part stays a few ulps of the high one, so nothing is lost against
-// folding after each addition, and the chain from one addition to the next is one FP32 addition.
-struct LazyDf {
-  float hi, lo;
-};
-__device__ __forceinline__ LazyDf red_add(LazyDf a, LazyDf b) {  // the same whichever operand comes first
-  const df s = two_sum(a.hi, b.hi);
-  return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
-}
-__device__ __forceinline__ LazyDf red_shfl_xor(LazyDf v, int o) {
-  return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-}
-__device__ __forceinline__ LazyDf red_shfl(LazyDf v, int src) {
-  return {__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
-}
-struct LazyRed {
-  using T = LazyDf;
-  static __device__ __forceinline__ T zero() { return {0.0f, 0.0f}; }
-  static __device__ __forceinline__ T sum(T v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v = red_add(v, red_shfl_xor(v, o));
-    return v;
-  }
-  static __device__ __forceinline__ float get(T v) { return __fadd_rn(v.hi, v.lo); }
-};
 
 // Two values of adjacent rows (or columns).
 struct Pair {
@@ -74,10 +47,9 @@ struct Pair {
 };
 
 // a.a b.a + a.b b.b
-__device__ __forceinline__ LazyDf dot(Pair a, Pair b) {
-  const float p = __fmul_rn(a.a, b.a), q = __fmul_rn(a.b, b.b);
-  const df s = two_sum(p, q);
-  return {s.hi, __fadd_rn(s.lo, __fadd_rn(__fmaf_rn(a.a, b.a, -p), __fmaf_rn(a.b, b.b, -q)))};
+__device__ __forceinline__ df dot(Pair a, Pair b) {
+  const float p = __fmul_rn(a.a, b.a);
+  return df_fma(df{p, __fmaf_rn(a.a, b.a, -p)}, a.b, b.b);
 }
 
 // (a.x b.x + c.x, a.y b.y + c.y), each rounded once as fmaf: one instruction for two FP32 multiply-adds.
@@ -186,7 +158,8 @@ __device__ __forceinline__ void stage_tiles(float *dst, const float *src, int nb
 
 
 template <int NX, int OP>
-__device__ void pcg_one_solve(const PcgArgs &a, const ProbDesc &d, float *sm, LazyDf *slots) {
+__device__ void pcg_one_solve(const PcgArgs &a, const ProbDesc &d, float *sm, df *slots) {
+  using Sum = Red<kRedDf, float>;
   constexpr int NXP = (NX + 3) & ~3;
   constexpr int H = (NX + 1) / 2;     // row pairs of a block row
   constexpr int LD4 = 4 * (H | 1);    // values of a tile row of an nx x nx block
@@ -321,9 +294,9 @@ __device__ void pcg_one_solve(const PcgArgs &a, const ProbDesc &d, float *sm, La
     }
   }
   r = g;
-  LazyDf g1[1] = {dot(g, g)};
-  block_sum<LazyRed, 1>(g1, slots);  // contains a barrier: staged blocks, reciprocals and sp complete
-  const float gg = LazyRed::get(g1[0]);
+  df g1[1] = {dot(g, g)};
+  block_sum<Sum, 1>(g1, slots);  // contains a barrier: staged blocks, reciprocals and sp complete
+  const float gg = Sum::get(g1[0]);
   const float thresh = a.tol2 * gg;
   const int max_iter = a.max_iter > 0 ? a.max_iter : 10 * n * NX;
   if (gg == 0.0f) {
@@ -353,11 +326,11 @@ __device__ void pcg_one_solve(const PcgArgs &a, const ProbDesc &d, float *sm, La
     // z = Phi^-1 r, r.z, r.r
     Pair z{0.0f, 0.0f};
     if (on) z = apply_P();
-    LazyDf s2[2] = {dot(r, z), dot(r, r)};
-    block_sum<LazyRed, 2>(s2, slots + 64);
+    df s2[2] = {dot(r, z), dot(r, r)};
+    block_sum<Sum, 2>(s2, slots + 64);
     const float rz_old = rz;
-    rz = LazyRed::get(s2[0]);
-    rr = LazyRed::get(s2[1]);
+    rz = Sum::get(s2[0]);
+    rr = Sum::get(s2[1]);
     if (first) {
       if (warm && a.warm == 2 && !(rr < gg)) {  // warm start no better than zero: restart from lambda_0 = 0
         warm = false;
@@ -384,9 +357,9 @@ __device__ void pcg_one_solve(const PcgArgs &a, const ProbDesc &d, float *sm, La
     // w = S p, p.w
     phase1(sp, pv, iq);
     if (on) w = apply_S(sp);
-    LazyDf s1v[1] = {dot(pv, w)};
-    block_sum<LazyRed, 1>(s1v, slots);
-    const float pw = LazyRed::get(s1v[0]);
+    df s1v[1] = {dot(pv, w)};
+    block_sum<Sum, 1>(s1v, slots);
+    const float pw = Sum::get(s1v[0]);
     if (!(pw > 0.0f) || !isfinite(pw)) { code = isfinite(pw) ? kBreakdown : kNonFinite; break; }
     const float alpha = rz / pw;
     x = {fmaf(alpha, pv.a, x.a), fmaf(alpha, pv.b, x.b)};
@@ -413,7 +386,7 @@ constexpr int one_min_ctas() { return NX <= 8 ? 2 : 1; }
 template <int NX, int OP>
 __global__ void __launch_bounds__(512, one_min_ctas<NX>()) pcg_one_kernel(PcgArgs a) {
   extern __shared__ float4 smem4[];
-  __shared__ __align__(16) LazyDf slots[4 * 32];
+  __shared__ __align__(16) df slots[4 * 32];
   __shared__ int s_next;
   for (int w = blockIdx.x;; w += gridDim.x) {
     if (a.counter) {
