@@ -219,7 +219,7 @@ struct NxGroup {
 struct sspcg_plan {
   int32_t nprob = 0;
   int mx = 1;       // largest nx and nu of the batch
-  int32_t max_nu = 0, max_N = 0;
+  int32_t max_nx = 1, max_nu = 0, max_N = 0;
   int mx_tiny = 1;  // of its FP64 subset
   std::vector<NxGroup> nxg_all, nxg_tiny;
   sspcg_options opts{};
@@ -794,6 +794,7 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     off_start[i + 1] = off_start[i] + Ni;
     all.push_back(i);
     p->mx = std::max(p->mx, std::max(nx[i], nu[i]));
+    p->max_nx = std::max(p->max_nx, nx[i]);
     p->max_nu = std::max(p->max_nu, nu[i]);
     p->max_N = std::max(p->max_N, N[i]);
     const bool f64 = opts->precision == SSPCG_PRECISION_F64 ||
@@ -1584,6 +1585,7 @@ PlanView plan_view(const sspcg_plan *p) {
   v.knot_start = p->knot_start.data();
   v.d_knot_start = p->d_knot_start;
   v.total_off = p->total_off;
+  v.max_nx = p->max_nx;
   v.max_nu = p->max_nu;
   v.max_N = p->max_N;
   return v;

@@ -78,7 +78,8 @@ struct LossArgs {
   double *uu, *gg, *loss;
   bf16 *dY;
 };
-cudaError_t launch_loss(const LossArgs &a, cudaStream_t st);
+// max_N, max_nx: bounds of the problems' sizes.
+cudaError_t launch_loss(const LossArgs &a, int max_N, int max_nx, cudaStream_t st, int sms);
 
 // Adam on the flat parameters from the splits of their gradients, whose sums go to g (update = false: only refresh the
 // bf16 copies).

@@ -302,7 +302,7 @@ sspcg_status sspcg_mlp_train_step(sspcg_mlp *n, const sspcg_plan *plan, int32_t 
   la.row0 = row0;
   la.Y = n->Y; la.lamstar = lambda_star; la.gamma = gamma; la.D = D; la.E = E;
   la.U = n->U; la.uu = n->uu; la.gg = n->gg; la.loss = loss; la.dY = n->dY;
-  MLP_CUDA(launch_loss(la, st));
+  MLP_CUDA(launch_loss(la, v.max_N, v.max_nx, st, host::sms()));
   // backward: output layer, then the two hidden layers (ReLU masks from the stored activations); the splits of the
   // gradients lie like the parameters
   float *part = n->part;

@@ -587,7 +587,15 @@ __global__ void __launch_bounds__(kColThreads) colsum_kernel(const bf16 *__restr
 // (S_{k,k-1} = E_{k-1} in the packed [N][nx][nx] layout, S_{k,k+1} = its
 // transpose); then dL/dlambda0 = 2 S u / (P ||gamma||^2).
 // ---------------------------------------------------------------------------
-constexpr int kLossThreads = 1024;  // a row per thread for most problems: a row is one chain of loads
+constexpr int kLossThreads = 1024;  // the widest CTA
+
+// Threads of a loss CTA for ``items`` rows or entries of the longest of P problems.  A row is one chain of loads, so a
+// few problems get a row per thread, up to 1024 (32 problems of 65 x 14 rows: the step 168 to 157 us); with more
+// problems than fit on the SMs at that width, 256 threads each, eight CTAs to an SM.
+int loss_block(int64_t items, int P, int sms) {
+  const int most = P <= 2 * sms ? kLossThreads : P <= 4 * sms ? 512 : 256;  // 2048 threads per SM
+  return (int)std::min<int64_t>(most, std::max<int64_t>(256, round_up(items, 32)));
+}
 
 // Sum over the CTA, for warp 0 (FP64 additions are too dear for every warp to repeat them).
 __device__ __forceinline__ double block_sum_d(double v, double *slots) {
@@ -801,11 +809,11 @@ cudaError_t launch_colsum(const bf16 *dY, const bf16 *dH2, const bf16 *dH1, int6
   return cudaGetLastError();
 }
 
-cudaError_t launch_loss(const LossArgs &a, cudaStream_t st) {
+cudaError_t launch_loss(const LossArgs &a, int max_N, int max_nx, cudaStream_t st, int sms) {
   const int P = a.p1 - a.p0;
   if (P <= 0) return cudaSuccess;
-  loss_u_kernel<<<P, kLossThreads, 0, st>>>(a);
-  loss_grad_kernel<<<P, kLossThreads, 0, st>>>(a);
+  loss_u_kernel<<<P, loss_block((int64_t)(max_N + 1) * max_nx, P, sms), 0, st>>>(a);
+  loss_grad_kernel<<<P, loss_block((int64_t)(max_N + 1) * kOut, P, sms), 0, st>>>(a);
   loss_total_kernel<<<1, 256, 0, st>>>(a.uu, a.gg, P, a.loss);
   return cudaGetLastError();
 }
