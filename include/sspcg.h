@@ -118,8 +118,9 @@ enum {
   SSPCG_SCHED_STREAM = 2,   /* operator and preconditioner read from L2/HBM every iteration */
   SSPCG_SCHED_WARP = 3,     /* plan calls: as RESIDENT, and every group of problems that fit whole in shared
                                memory (QP operator form, textbook PCG, double-float or FP64 sums) runs one
-                               problem per warp, as many warps per CTA as fit (at most 16); other entry
-                               points: as RESIDENT */
+                               problem per warp, as many warps per CTA as fit (at most 16); the few sizes
+                               that fit whole in the smaller layout of the row-pair kernel only (see
+                               sspcg_plan_create) run there; other entry points: as RESIDENT */
 };
 
 /* Solver options. */
@@ -263,7 +264,12 @@ sspcg_status sspcg_residual_qp(int32_t N, int32_t nx, int32_t nu, const float *A
  * one device buffer per array kind, each problem starting at a 16-byte
  * aligned offset given by sspcg_plan_offsets.  The plan owns its device
  * descriptors and work lists (allocated here, freed by sspcg_plan_destroy)
- * and picks a kernel schedule per problem class.  It also holds padded
+ * and picks a kernel schedule per problem class: FP32 problems that fit in
+ * shared memory whole and have at most 512 pairs of rows take the row-pair
+ * kernel (a thread per two adjacent rows; textbook PCG, double-float sums,
+ * degree 0, any schedule but STREAM), the others the general kernel.  Both
+ * form the same block products; their dot products group the same terms
+ * differently, so results agree to rounding.  It also holds padded
  * copies of A, B and PE for the problems that do not fit in shared memory
  * whole (every problem under SSPCG_SCHED_STREAM): about N nx (2 nx4 + nu4) floats
  * each, with nx4 and nu4 rounded up to multiples of 4.  The QP-form batched

@@ -177,6 +177,7 @@ struct PcgGroup {
   bool stream = false;       // stage no block rows (the schedule option, or the tuner's choice)
   int share = 1;             // partially staged groups: stage into 1/share of the shared memory (tuner's choice)
   bool one = false;          // a thread per row pair (one_fits for every member)
+  bool pairs_only = false;   // WARP schedule: members that the general kernel, warps included, holds only in part
   int warps = 0;             // > 0: one problem per warp, this many warps per CTA (tuner's choice; see warp_ok)
   bool tuned = false;        // block and residency from the tuner (this plan's, or its cache)
   int64_t slot_elems = 0, scratch_off = 0;
@@ -357,7 +358,7 @@ TuneKey tune_key(const sspcg_plan *p, const GroupSet &set, const PcgGroup &g) {
 // One problem per warp exists for fully staged groups of the QP form with textbook PCG: the FP64 path, and
 // FP32 with double-float sums.
 bool warp_ok(const sspcg_plan *p, const GroupSet &set, const PcgGroup &g) {
-  if (set.op != kOpQp || g.gvec || g.cls < 1 || g.cls > 4) return false;
+  if (set.op != kOpQp || g.gvec || g.pairs_only || g.cls < 1 || g.cls > 4) return false;
   if (set.f64) return true;
   return red_mode(p->opts.reduction) == kRedDf && p->opts.cg_variant == 0;
 }
@@ -380,6 +381,7 @@ sspcg_status shape_group(const sspcg_plan *p, const GroupSet &set, PcgGroup &g, 
       const int sched = g.stream ? SSPCG_SCHED_STREAM : p->opts.schedule;
       if (!pcg_fit(set.op, sched, d.N, d.nx, d.nu, set.f64, p->opts.poly_degree, cg, &K, &b, g.stream ? 1 : g.share))
         return SSPCG_ERR_UNSUPPORTED;
+      if (g.warps > 0 && K <= d.N) return SSPCG_ERR_UNSUPPORTED;  // a warp's problem is staged whole
     }
     maxbytes = std::max(maxbytes, b);
   }
@@ -420,16 +422,22 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
   // class 0: not fully resident (takes the whole budget); classes 1..3: fully resident within
   // budget/2, /4, /8 (several CTAs per SM); class 4: the rest of the fully resident problems
   // class 5: vectors in a global workspace (they alone exceed the shared memory)
-  // each class split into the problems that run with a thread per row pair and the others
-  constexpr int kClasses = 6;
-  std::vector<std::vector<int32_t>> buckets(2 * kClasses * (kMaxNx + 1));
+  // each class split by kind: 0 general kernel, 1 a thread per row pair, 2 the same for problems that fit whole in its
+  // layout only, which a plan of the WARP schedule keeps from those that run one per warp
+  constexpr int kClasses = 6, kKinds = 3;
+  std::vector<std::vector<int32_t>> buckets(kKinds * kClasses * (kMaxNx + 1));
   std::vector<int64_t> bytes(descs.size(), 0);
   const int64_t budget = smem_budget();
   for (int32_t i : members) {
     const ProbDesc &d = descs[i];
     int K = 0;
     const bool one = one_fits(set.op, &p->opts, set.f64, d.N, d.nx, d.nu);
+    int kind = one ? 1 : 0;
     if (one) {
+      if (p->opts.schedule == SSPCG_SCHED_WARP && set.op == kOpQp &&
+          !(pcg_fit(set.op, p->opts.schedule, d.N, d.nx, d.nu, false, p->opts.poly_degree, p->opts.cg_variant, &K,
+                    &bytes[i]) && K > d.N))
+        kind = 2;
       K = d.N + 1;
       bytes[i] = pcg_one_layout(set.op, d.N, d.nx, d.nu).total * (int64_t)sizeof(float);
     } else if (!pcg_fit(set.op, p->opts.schedule, d.N, d.nx, d.nu, set.f64, p->opts.poly_degree, p->opts.cg_variant, &K,
@@ -438,7 +446,7 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
         set.unsupported = true;
         continue;
       }
-      buckets[2 * (kClasses * d.nx + 5)].push_back(i);
+      buckets[kKinds * (kClasses * d.nx + 5)].push_back(i);
       continue;
     }
     int cls = 0;
@@ -446,12 +454,12 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
       const int64_t need = bytes[i] + kPcgStaticSmem + 1024;
       cls = need * 8 <= budget ? 3 : need * 4 <= budget ? 2 : need * 2 <= budget ? 1 : 4;
     }
-    buckets[2 * (kClasses * d.nx + cls) + (one ? 1 : 0)].push_back(i);
+    buckets[kKinds * (kClasses * d.nx + cls) + kind].push_back(i);
   }
   for (int nx = 1; nx <= kMaxNx; ++nx) {
-    for (int rb = 0; rb < 2 * kClasses; ++rb) {
-      const int r = rb / 2;
-      auto &b = buckets[2 * kClasses * nx + rb];
+    for (int rb = 0; rb < kKinds * kClasses; ++rb) {
+      const int r = rb / kKinds;
+      auto &b = buckets[kKinds * kClasses * nx + rb];
       if (b.empty()) continue;
       std::stable_sort(b.begin(), b.end(), [&](int32_t x, int32_t y) { return descs[x].N > descs[y].N; });
       PcgGroup g;
@@ -459,7 +467,8 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
       g.cls = r;
       g.resident = r != 0 && r != 5;
       g.gvec = r == 5;
-      g.one = rb % 2 == 1;
+      g.one = rb % kKinds > 0;
+      g.pairs_only = rb % kKinds == 2;
       g.f64 = set.f64;
       g.stream = p->opts.schedule == SSPCG_SCHED_STREAM;
       g.members = b;
@@ -488,10 +497,9 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
         int64_t slot = 0;
         for (int32_t i : b) {
           int K = 0;
-          int64_t need = 0;
-          if (!pcg_fit(set.op, SSPCG_SCHED_RESIDENT, descs[i].N, nx, descs[i].nu, set.f64, p->opts.poly_degree,
-                       p->opts.cg_variant, &K, &need))
-            need = smem_budget();
+          int64_t need = 0;  // of the general kernel's layout, which holds the members whole
+          pcg_fit(set.op, p->opts.schedule, descs[i].N, nx, descs[i].nu, set.f64, p->opts.poly_degree,
+                  p->opts.cg_variant, &K, &need);
           slot = std::max(slot, round_up(need, 16));
         }
         const int64_t fit = slot > 0 ? smem_budget() / slot : 1;
