@@ -408,17 +408,18 @@ sspcg_status sspcg_plan_launch(sspcg_plan *plan, sspcg_stream stream);
  * sspcg_pipeline_batched, then, for every PCG launch group of the chosen
  * sets (which: SSPCG_TUNE_PIPELINE, the pipeline's FP32 and FP64 sets;
  * SSPCG_TUNE_SOLVE, the set of sspcg_solve_qp_batched; or both; one group
- * per nx and residency class), times candidate schedules alone on these
- * inputs: block sizes 64..512 threads (16 rows per thread to one); for
- * groups that do not fit in shared memory whole, staging the first rows into
- * the whole budget or into 1/2, 1/3 or 1/4 of it (several CTAs per SM), or
- * streaming every block row from L2; for groups that do fit (QP form,
+ * per nx, residency class and kernel), times candidate schedules alone on
+ * these inputs: for groups of the general kernel, block sizes 64..512 threads
+ * (16 rows per thread to one; the row-pair kernel takes a thread per pair);
+ * for groups that do not fit in shared memory whole, staging the first rows
+ * into the whole budget or into 1/2, 1/3 or 1/4 of it (several CTAs per SM),
+ * or streaming every block row from L2; for groups that do fit (QP form,
  * textbook PCG, double-float or FP64 sums), also one problem per warp with
  * 1 to 16 warps per CTA.  Each group keeps its fastest
  * candidate (grid from the kernel's occupancy at that block size); the
  * choices also go to a process-wide cache keyed by (launch set, operator form,
  * precision, reduction, polynomial degree, PCG variant, nx, residency class,
- * bucket of the largest N: <16, <32, ..., <512, >=512), which later
+ * kernel, bucket of the largest N: <16, <32, ..., <512, >=512), which later
  * sspcg_plan_create calls with block_threads = 0 and the automatic schedule
  * apply to matching groups.  Costs about 30 launches of each group.
  * Arguments as sspcg_pipeline_batched; lambda, iters and relres are
@@ -445,7 +446,8 @@ sspcg_status sspcg_plan_autotune(sspcg_plan *plan, int32_t which, sspcg_precond 
  * tuner or its cache (0/1), shared-memory share (a partially staged group
  * stages into 1/share of the budget, so up to share CTAs fit on an SM),
  * warps per CTA when each warp solves its own problem (0: one problem per
- * CTA).
+ * CTA).  The rows do not say which kernel a group of one problem per CTA
+ * runs; sspcg_plan_create does.
  */
 sspcg_status sspcg_plan_schedule(const sspcg_plan *plan, int32_t which, int32_t *out, int32_t capacity,
                                  int32_t *count);

@@ -363,6 +363,11 @@ bool warp_ok(const sspcg_plan *p, const GroupSet &set, const PcgGroup &g) {
   return red_mode(p->opts.reduction) == kRedDf && p->opts.cg_variant == 0;
 }
 
+// Threads per CTA of a group whose CTAs take one problem each.
+int group_block(const sspcg_plan *p, const PcgGroup &g) {
+  return p->opts.block_threads > 0 ? p->opts.block_threads : g.one ? one_block(g.maxN, g.nx) : auto_block(g.maxrows);
+}
+
 // Dynamic shared memory, slot size and grid of a group for its block size and residency: every member's
 // layout (K = 0 when streaming), CTAs per SM from the kernel's occupancy (registers, threads, shared memory).
 sspcg_status shape_group(const sspcg_plan *p, const GroupSet &set, PcgGroup &g, const std::vector<ProbDesc> &descs) {
@@ -479,7 +484,7 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
         // bytes per iteration times iterations, which grow about as sqrt(N + 1)
         g.work += std::pow((double)(d.N + 1), 1.5) * d.nx * (3.0 * d.nx + d.nu);
       }
-      g.block = p->opts.block_threads > 0 ? p->opts.block_threads : g.one ? one_block(g.maxN, nx) : auto_block(g.maxrows);
+      g.block = group_block(p, g);
       g.nwork = (int32_t)b.size();
       if (p->opts.block_threads == 0 && p->opts.schedule == SSPCG_SCHED_AUTO) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -519,8 +524,7 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
       sspcg_status s = shape_group(p, set, g, descs);
       if (s == SSPCG_ERR_UNSUPPORTED && g.warps > 0) {  // a warp count whose slots do not fit this group
         g.warps = 0;
-        if (p->opts.block_threads == 0) g.block = g.one ? one_block(g.maxN, nx) : auto_block(g.maxrows);
-        else g.block = p->opts.block_threads;
+        g.block = group_block(p, g);
         s = shape_group(p, set, g, descs);
       }
       if (s != SSPCG_OK) return s;
@@ -1297,11 +1301,22 @@ sspcg_status tune_set(sspcg_plan *p, GroupSet &set, const std::vector<ProbDesc> 
                       const int32_t *status0, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
   static const int kBlocks[] = {64, 96, 128, 160, 192, 256, 320, 384, 448, 512};
   for (PcgGroup &g : set.groups) {
-    const PcgGroup orig = g;
+    PcgGroup orig = g;
     float best_ms = 0.0f;
     sspcg_status s = time_group(p, set, g, base, status0, st, e0, e1, &best_ms);
     if (s != SSPCG_OK) return s;
     PcgGroup best = g;
+    if (g.warps > 0) {  // one problem per warp by the cache or the schedule: the CTA candidates start from the default
+      orig.warps = 0;
+      orig.block = group_block(p, orig);
+      if ((s = shape_group(p, set, orig, descs)) != SSPCG_OK) return s;
+      float ms = 0.0f;
+      if ((s = time_group(p, set, orig, base, status0, st, e0, e1, &ms)) != SSPCG_OK) return s;
+      if (ms < best_ms) {
+        best_ms = ms;
+        best = orig;
+      }
+    }
     // from at most 16 rows per thread to at most one
     const int64_t max_block = std::max<int64_t>(64, round_up(g.maxrows, 32));
     const int64_t min_block = std::min<int64_t>(max_block, g.maxrows / 16);
