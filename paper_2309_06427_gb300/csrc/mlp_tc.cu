@@ -7,7 +7,8 @@
 // releases each stage with tcgen05.commit; then all four warps read the
 // accumulators (tcgen05.ld, one TMEM lane per row) and apply the epilogue.
 // Every mbarrier wait is bounded: on expiry the kernel records an error code,
-// skips its remaining work, frees its tensor memory and returns.
+// skips its remaining work, waits (bounded again) for its copies and products
+// in flight, frees its tensor memory and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -20,7 +21,11 @@ namespace {
 constexpr int kTcM = 128;          // rows per tile (TMEM lanes)
 constexpr int kTcK = 64;           // columns per stage: one 128-byte swizzle row of bf16
 constexpr int kTcThreads = 128;
-constexpr uint32_t kSpinLimit = 1u << 26;  // polls of one mbarrier wait (well over a second)
+#ifndef SSPCG_TC_POLLS
+#define SSPCG_TC_POLLS (1u << 26)
+#endif
+constexpr uint32_t kSpinLimit = SSPCG_TC_POLLS;  // polls of one mbarrier wait (well over a second)
+constexpr uint32_t kDrainLimit = 1u << 26;       // of the waits that follow one that ran out
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
@@ -33,9 +38,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
 }
 
 // Wait until the phase of parity ``parity`` has completed; false when the bound expires.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit = kSpinLimit) {
   const uint32_t a = su32(bar);
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+  for (uint32_t i = 0; i < limit; ++i) {
     uint32_t done;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -149,6 +154,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  int issued = 0;  // the producer's stages on their way
 
   if (warp == 0 && lane == 0) {
     // producer: TMA loads of A rows [m0, m0 + 128 MT) and B rows [n0, n0 + N), 64 columns per stage
@@ -165,6 +171,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       for (int t = 0; t < MT; ++t)
         tma_load_2d(a + t * (C::kABytes / MT), &mapA, kt * kTcK, (int)m0 + t * kTcM, &full[s]);
       tma_load_2d(b, &mapB, kt * kTcK, n0, &full[s]);
+      issued = kt + 1;
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
@@ -227,6 +234,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
       }
     }
+  } else if (threadIdx.x == 0) {  // what is in flight ends before the shared and the tensor memory go
+    for (int kt = issued > C::kStages ? issued - C::kStages : 0; kt < issued; ++kt)
+      mbar_wait(&full[kt % C::kStages], (kt / C::kStages) & 1, kDrainLimit);
+    mbar_wait(acc_full, 0, kDrainLimit);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -300,11 +311,12 @@ __global__ void __launch_bounds__(kTailThreads, 1)
   const uint32_t tmem = tmem_slot, acc3 = tmem + kHid;  // accumulators: columns 0-255 and 256-287
   const int quarter = warp & 3, r = quarter * 32 + lane;
   const uint32_t tlane = (uint32_t)(quarter * 32) << 16;
-  bool ok = true;
+  bool ok = true, second = false, third = false;  // thread 0: this tile's products have been issued
   uint32_t parity = 0;
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, parity ^= 1) {
     if (first) {
-      ok = mbar_wait(&bar_w, 0) && mbar_wait(&bar_a, parity);
+      third = false;
+      second = ok = mbar_wait(&bar_w, 0) && mbar_wait(&bar_a, parity);
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         for (int kt = 0; kt < kTailKT; ++kt)
@@ -354,6 +366,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
           mma_issue(acc3, smem_desc(sA + kt * kTailABytes + k * 32), smem_desc(sW3 + kt * kTailW3Bytes + k * 32),
                     instr_desc(kTcM, kOut), (kt > 0 || k > 0) ? 1u : 0u);
       mma_commit(&bar_3);
+      third = true;
     }
     __syncwarp();
     ok = __all_sync(0xffffffffu, mbar_wait(&bar_3, parity));
@@ -378,6 +391,12 @@ __global__ void __launch_bounds__(kTailThreads, 1)
           if (i < d.nx) o[i] = v[i] + __ldg(b3 + i);
       }
     }
+  }
+  if (first && !ok) {  // what is in flight ends before the shared and the tensor memory go
+    mbar_wait(&bar_w, 0, kDrainLimit);
+    mbar_wait(&bar_a, parity, kDrainLimit);
+    if (second) mbar_wait(&bar_2, parity, kDrainLimit);
+    if (third) mbar_wait(&bar_3, parity, kDrainLimit);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
