@@ -663,7 +663,7 @@ sspcg_status sspcg_build_schur(int32_t N, int32_t nx, int32_t nu, const float *A
   if (!shape_ok(N, nx, nu)) return SSPCG_ERR_INVALID_ARG;
   if (!qd || !D || (N > 0 && (!A || !rd || !E || (nu > 0 && !B)))) return SSPCG_ERR_INVALID_ARG;
   ProbSet ps{nullptr, single_desc(N, nx, nu), 1};
-  SSPCG_CUDA(launch_schur_f32(ps, N, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
+  SSPCG_CUDA(launch_schur_f32(ps, N, nx, nu, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
   return SSPCG_OK;
 }
 
@@ -698,7 +698,7 @@ sspcg_status sspcg_build_precond(int32_t N, int32_t nx, sspcg_precond kind, cons
   ProbSet ps{nullptr, single_desc(N, nx, 0), 1};
   SSPCG_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
   SSPCG_CUDA(launch_precond_inv<float>(ps, nullptr, N + 1, nx, (int)kind, D, PD, status, st));
-  SSPCG_CUDA(launch_precond_off_f32(ps, N, (int)kind, E, PD, PE, st, device_sms(), (int64_t)N * nx * nx));
+  SSPCG_CUDA(launch_precond_off_f32(ps, N, nx, (int)kind, E, PD, PE, st, device_sms(), (int64_t)N * nx * nx));
   return SSPCG_OK;
 }
 
@@ -986,7 +986,8 @@ sspcg_status sspcg_build_schur_batched(sspcg_plan *plan, const float *A, const f
   if (plan->nprob == 0) return SSPCG_OK;
   if (!qd || !D || !aligned16(qd) || !aligned16(D)) return SSPCG_ERR_INVALID_ARG;
   if (plan->total_off > 0 && (!A || !rd || !E || !B)) return SSPCG_ERR_INVALID_ARG;
-  SSPCG_CUDA(launch_schur_f32(plan_set(plan), plan->max_N, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
+  SSPCG_CUDA(launch_schur_f32(plan_set(plan), plan->max_N, plan->max_nx, plan->max_nu, A, B, qd, rd, D, E,
+                              (cudaStream_t)stream, device_sms()));
   return SSPCG_OK;
 }
 
@@ -1075,8 +1076,8 @@ sspcg_status sspcg_build_precond_batched(sspcg_plan *plan, sspcg_precond kind, c
   for (const NxGroup &g : plan->nxg_all)
     SSPCG_CUDA(launch_precond_inv<float>(ProbSet{g.d_desc, ProbDesc{}, g.nprob}, g.d_refs, g.knots, g.nx,
                                          (int)kind, D, PD, status, st));
-  SSPCG_CUDA(launch_precond_off_f32(plan_set(plan), plan->max_N, (int)kind, E, PD, PE, st, device_sms(),
-                                    plan->sizes[SSPCG_ARRAY_OFF]));
+  SSPCG_CUDA(launch_precond_off_f32(plan_set(plan), plan->max_N, plan->max_nx, (int)kind, E, PD, PE, st,
+                                    device_sms(), plan->sizes[SSPCG_ARRAY_OFF]));
   return SSPCG_OK;
 }
 

@@ -46,16 +46,17 @@ __host__ __device__ __forceinline__ int schur_chunk(int nx, int nu) {
   return by_tiles < by_smem ? by_tiles : by_smem;
 }
 
-__global__ void __launch_bounds__(kSchurThreads) schur_f32_kernel(ProbSet ps, int per, const float *__restrict__ A,
+__global__ void __launch_bounds__(kSchurThreads) schur_f32_kernel(ProbSet ps, ChunkSplit split,
+                                                                  const float *__restrict__ A,
                                                                   const float *__restrict__ B,
                                                                   const float *__restrict__ qd,
                                                                   const float *__restrict__ rd, float *__restrict__ D,
                                                                   float *__restrict__ E) {
   __shared__ __align__(16) float sm[kSchurFloats];
   const int tid = threadIdx.x;
-  const ProbDesc d = ps.get(blockIdx.x / per);
+  const ProbDesc d = ps.get(blockIdx.x / split.per);
   const int N = d.N, nx = d.nx, nu = d.nu, nn = nx * nx, m = nx + nu, nt = tiles4(nx), ld = 4 * nt;
-  const int ntl = nt * (nt + 1) / 2, C = chunk_share(schur_chunk(nx, nu), N, per);
+  const int ntl = nt * (nt + 1) / 2, per = split.per, C = chunk_length(schur_chunk(nx, nu), N, split.share);
   const Divisor by_nx(nx), by_nu(nu), by_ntl(ntl);
   const int part = blockIdx.x % per;
   if (part == 0) {
@@ -134,15 +135,15 @@ __host__ __device__ __forceinline__ int off_chunk(int nx) {
   return by_tiles < by_smem ? by_tiles : by_smem;
 }
 
-__global__ void __launch_bounds__(kOffThreads, 4) precond_off_f32_kernel(ProbSet ps, int per, float c,
+__global__ void __launch_bounds__(kOffThreads, 4) precond_off_f32_kernel(ProbSet ps, ChunkSplit split, float c,
                                                                       const float *__restrict__ E,
                                                                       const float *__restrict__ PD,
                                                                       float *__restrict__ PE) {
   __shared__ __align__(16) float sm[kOffFloats];
   const int tid = threadIdx.x;
-  const ProbDesc d = ps.get(blockIdx.x / per);
+  const ProbDesc d = ps.get(blockIdx.x / split.per);
   const int N = d.N, nx = d.nx, nn = nx * nx, nt = tiles4(nx), ld = 4 * nt, blk = nx * ld, ntl = nt * nt;
-  const int C = chunk_share(off_chunk(nx), N, per);
+  const int per = split.per, C = chunk_length(off_chunk(nx), N, split.share);
   const Divisor by_ntl(ntl), by_nt(nt);
   for (int b0 = (int)(blockIdx.x % per) * C; b0 < N; b0 += per * C) {
     const int nb = min(C, N - b0);
@@ -188,28 +189,24 @@ __global__ void __launch_bounds__(kOffThreads, 4) precond_off_f32_kernel(ProbSet
   }
 }
 
-// CTAs per problem: enough for ``want`` on every SM, no more than the longest problem has chunks of 3 blocks.
-int ctas_per_problem(const ProbSet &ps, int max_N, int want, int sms) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>(cdiv((int64_t)want * sms, ps.nprob), cdiv(max_N, 3)));
-}
-
 }  // namespace
 
-cudaError_t launch_schur_f32(const ProbSet &ps, int max_N, const float *A, const float *B, const float *qd,
-                             const float *rd, float *D, float *E, cudaStream_t st, int sms) {
+cudaError_t launch_schur_f32(const ProbSet &ps, int max_N, int max_nx, int max_nu, const float *A,
+                             const float *B, const float *qd, const float *rd, float *D, float *E, cudaStream_t st, int sms) {
   if (ps.nprob == 0) return cudaSuccess;
-  const int per = ctas_per_problem(ps, max_N, 40, sms);
-  schur_f32_kernel<<<(unsigned)ps.nprob * per, kSchurThreads, 0, st>>>(ps, per, A, B, qd, rd, D, E);
+  const ChunkSplit split = chunk_split(ps.nprob, sms, max_N, schur_chunk(max_nx, max_nu), 3);
+  schur_f32_kernel<<<(unsigned)ps.nprob * split.per, kSchurThreads, 0, st>>>(ps, split, A, B, qd, rd, D, E);
   return cudaGetLastError();
 }
 
-cudaError_t launch_precond_off_f32(const ProbSet &ps, int max_N, int kind, const float *E, const float *PD, float *PE,
-                                   cudaStream_t st, int sms, int64_t off_elems) {
+cudaError_t launch_precond_off_f32(const ProbSet &ps, int max_N, int max_nx, int kind, const float *E,
+                                   const float *PD, float *PE, cudaStream_t st, int sms, int64_t off_elems) {
   if (off_elems == 0 || max_N == 0) return cudaSuccess;
   if (kind == 2 || kind == 3)  // block-Jacobi, Jacobi: no off-diagonal blocks
     return cudaMemsetAsync(PE, 0, sizeof(float) * off_elems, st);
-  const int per = ctas_per_problem(ps, max_N, 32, sms);
-  precond_off_f32_kernel<<<(unsigned)ps.nprob * per, kOffThreads, 0, st>>>(ps, per, kind == 0 ? 1.0f : 0.5f, E, PD, PE);
+  const ChunkSplit split = chunk_split(ps.nprob, sms, max_N, off_chunk(max_nx), 3);
+  precond_off_f32_kernel<<<(unsigned)ps.nprob * split.per, kOffThreads, 0, st>>>(ps, split, kind == 0 ? 1.0f : 0.5f, E,
+                                                                                 PD, PE);
   return cudaGetLastError();
 }
 

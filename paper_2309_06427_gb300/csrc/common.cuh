@@ -144,10 +144,35 @@ __host__ __device__ __forceinline__ int chunk_rows(int nx, int nu) {
   return c > 64 ? 64 : c;
 }
 
-// Block rows (or blocks) per chunk when ``per`` CTAs share ``rows`` of a problem: a lone problem goes to all of them in
-// short chunks instead of to a few in full ones (nx = 14, N = 103, build and solve: 681 to 677 us).
-__device__ __forceinline__ int chunk_share(int full, int rows, int per) {
-  return min(full, max(1, (rows + per - 1) / per));
+// CTAs of a launch over chunks: ``per`` for every problem, which is cut into ``share`` chunks at least.
+struct ChunkSplit {
+  int per, share;
+};
+
+// The split of nprob problems of at most ``rows`` block rows; full: rows of a full chunk of the largest blocks; least:
+// rows that a CTA is worth.  A CTA costs as much as some ten rows of small blocks, so problems are cut into shorter
+// chunks only while all CTAs run at once, three to an SM: a lone problem goes to many CTAs (nx = 14, N = 103, build and
+// solve: 681 to 677 us), 304 problems of 64 rows to one each.  (Seven CTAs to an SM are slower at 64 problems of 64 rows,
+// one or two on few long problems.  Cutting without regard to what runs at once made the 304 problems' Schur blocks of
+// nx = 4 take 30 us for 6, the right-hand side of 512 problems of 20 rows 11 us for 5.)  Longer problems get a CTA per
+// full chunk, up to 56 CTAs per SM in all: the largest of a mixed batch of 4096 end it (two CTAs each, primal steps: 133
+// us for 158), and CTAs that find no chunk cost the more the more problems are small.
+inline ChunkSplit chunk_split(int64_t nprob, int sms, int rows, int full, int least) {
+  if (rows < 1 || nprob < 1) return {1, 1};
+  int64_t share = 3 * (int64_t)sms / nprob;
+  if (share > cdiv(rows, least)) share = cdiv(rows, least);
+  if (share < 1) share = 1;
+  int64_t per = 56 * (int64_t)sms / nprob;
+  if (per > cdiv(rows, full)) per = cdiv(rows, full);
+  if (per < share) per = share;
+  return {(int)per, (int)share};
+}
+
+// Rows per chunk of a problem.
+__host__ __device__ __forceinline__ int chunk_length(int full, int rows, int share) {
+  if (share < 2) return full;  // no division: short kernels notice it
+  const int c = (rows + share - 1) / share;
+  return c < 1 ? 1 : c < full ? c : full;
 }
 
 // Quotients by a divisor d <= 64 known at run time, for e < 2^20: the high word of e times ceil(2^32 / d), whose

@@ -211,11 +211,11 @@ template <typename Real>
 cudaError_t launch_schur_build(const ProbSet &ps, const int2 *refs, int64_t total_knots, const float *A,
                                const float *B, const float *qd, const float *rd, Real *D, Real *E,
                                cudaStream_t st, int sms, int mx);
-// The same in FP32 (build_f32.cu); max_N: the largest horizon of the set; off_elems: values of PE.
-cudaError_t launch_schur_f32(const ProbSet &ps, int max_N, const float *A, const float *B, const float *qd,
-                             const float *rd, float *D, float *E, cudaStream_t st, int sms);
-cudaError_t launch_precond_off_f32(const ProbSet &ps, int max_N, int kind, const float *E, const float *PD, float *PE,
-                                   cudaStream_t st, int sms, int64_t off_elems);
+// The same in FP32 (build_f32.cu); max_N, max_nx, max_nu: the largest sizes of the set; off_elems: values of PE.
+cudaError_t launch_schur_f32(const ProbSet &ps, int max_N, int max_nx, int max_nu, const float *A, const float *B,
+                             const float *qd, const float *rd, float *D, float *E, cudaStream_t st, int sms);
+cudaError_t launch_precond_off_f32(const ProbSet &ps, int max_N, int max_nx, int kind, const float *E, const float *PD,
+                                   float *PE, cudaStream_t st, int sms, int64_t off_elems);
 // Schur blocks with full SPD cost blocks from their inverses: Qi laid out like
 // D, R_{k-1}^-1 of problem p at roff[p] + (k-1) nu^2 (roff nullptr: offset 0).
 cudaError_t launch_schur_full(const ProbSet &ps, const int2 *refs, int64_t total_knots, const int64_t *roff,

@@ -26,17 +26,17 @@ namespace {
 
 constexpr int kKktThreads = 256;
 
-// CTA b takes chunks b % per, b % per + per, ... of problem b / per.
-__global__ void __launch_bounds__(kKktThreads)
-    form_gamma_kernel(ProbSet ps, int per, const float *__restrict__ A, const float *__restrict__ B,
+// With ``per`` CTAs for each problem, CTA b takes chunks b % per, b % per + per, ... of problem b / per.
+__global__ void __launch_bounds__(kKktThreads, 7)  // what the shared memory holds; five CTAs take a quarter longer
+    form_gamma_kernel(ProbSet ps, ChunkSplit split, const float *__restrict__ A, const float *__restrict__ B,
                       const float *__restrict__ qd, const float *__restrict__ rd, const float *__restrict__ c,
                       const float *__restrict__ q, const float *__restrict__ r, float *__restrict__ gamma) {
   __shared__ float sm[kChunkFloats];
   __shared__ float sg[kChunkItems + kMaxNx];  // scaled gradients q_k / qd_k, r_k / rd_k, nx + nu per block
   const int tid = threadIdx.x;
-  const ProbDesc d = ps.get(blockIdx.x / per);
-  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu,
-            C = chunk_share(chunk_rows(nx, nu), N + 1, per);
+  const ProbDesc d = ps.get(blockIdx.x / split.per);
+  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu, per = split.per,
+            C = chunk_length(chunk_rows(nx, nu), N + 1, split.share);
   const int lda = nx | 1, ldb = nu | 1;
   const Divisor by_m(m), by_nx(nx);
   float *sA = sm, *sB = sm + C * nx * lda;
@@ -69,15 +69,15 @@ __global__ void __launch_bounds__(kKktThreads)
 }
 
 __global__ void __launch_bounds__(kKktThreads)
-    recover_step_kernel(ProbSet ps, int per, const float *__restrict__ A, const float *__restrict__ B,
+    recover_step_kernel(ProbSet ps, ChunkSplit split, const float *__restrict__ A, const float *__restrict__ B,
                         const float *__restrict__ qd, const float *__restrict__ rd, const float *__restrict__ q,
                         const float *__restrict__ r, const float *__restrict__ mu, float *__restrict__ dx,
                         float *__restrict__ du) {
   __shared__ float sm[kChunkItems + kMaxNx];  // mu_{k+1} of the chunk's block rows
   const int tid = threadIdx.x;
-  const ProbDesc d = ps.get(blockIdx.x / per);
-  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu,
-            C = chunk_share(chunk_rows(nx, nu), N + 1, per);
+  const ProbDesc d = ps.get(blockIdx.x / split.per);
+  const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu, per = split.per,
+            C = chunk_length(chunk_rows(nx, nu), N + 1, split.share);
   const Divisor by_m(m);
   for (int k0 = (int)(blockIdx.x % per) * C; k0 <= N; k0 += per * C) {
     const int k1 = min(N + 1, k0 + C), nb = min(k1, N) - k0;
@@ -114,10 +114,8 @@ __global__ void __launch_bounds__(kKktThreads)
   }
 }
 
-// CTAs per problem: enough for 16 on every SM, no more than the longest problem has chunks (at least 4 block rows).
-int kkt_per(int64_t nprob, int64_t max_N) {
-  const int64_t want = cdiv((int64_t)16 * host::sms(), nprob), most = cdiv(max_N + 1, 4);
-  return (int)std::max<int64_t>(1, std::min(want, most));
+ChunkSplit kkt_split(int64_t nprob, int max_N, int nx, int nu) {
+  return chunk_split(nprob, host::sms(), max_N + 1, chunk_rows(nx, nu), 4);
 }
 
 bool shape_ok(int N, int nx, int nu) {
@@ -148,8 +146,8 @@ sspcg_status sspcg_form_gamma(int32_t N, int32_t nx, int32_t nu, const float *A,
                               sspcg_stream stream) {
   if (!shape_ok(N, nx, nu)) return SSPCG_ERR_INVALID_ARG;
   if (!qd || !c || !q || !gamma || (N > 0 && (!A || (nu > 0 && (!B || !rd || !r))))) return SSPCG_ERR_INVALID_ARG;
-  const int per = kkt_per(1, N);
-  form_gamma_kernel<<<per, kKktThreads, 0, (cudaStream_t)stream>>>(ProbSet{nullptr, single(N, nx, nu), 1}, per, A, B, qd,
+  const ChunkSplit split = kkt_split(1, N, nx, nu);
+  form_gamma_kernel<<<split.per, kKktThreads, 0, (cudaStream_t)stream>>>(ProbSet{nullptr, single(N, nx, nu), 1}, split, A, B, qd,
                                                                    rd, c, q, r, gamma);
   KKT_CUDA(cudaGetLastError());
   return SSPCG_OK;
@@ -161,8 +159,8 @@ sspcg_status sspcg_recover_step(int32_t N, int32_t nx, int32_t nu, const float *
   if (!shape_ok(N, nx, nu)) return SSPCG_ERR_INVALID_ARG;
   if (!qd || !q || !mu || !dx || (N > 0 && (!A || (nu > 0 && (!B || !rd || !r || !du)))))
     return SSPCG_ERR_INVALID_ARG;
-  const int per = kkt_per(1, N);
-  recover_step_kernel<<<per, kKktThreads, 0, (cudaStream_t)stream>>>(ProbSet{nullptr, single(N, nx, nu), 1}, per, A, B,
+  const ChunkSplit split = kkt_split(1, N, nx, nu);
+  recover_step_kernel<<<split.per, kKktThreads, 0, (cudaStream_t)stream>>>(ProbSet{nullptr, single(N, nx, nu), 1}, split, A, B,
                                                                      qd, rd, q, r, mu, dx, du);
   KKT_CUDA(cudaGetLastError());
   return SSPCG_OK;
@@ -175,8 +173,8 @@ sspcg_status sspcg_form_gamma_batched(sspcg_plan *plan, const float *A, const fl
   const host::PlanView v = host::plan_view(plan);
   if (v.nprob == 0) return SSPCG_OK;
   if (!qd || !c || !q || !gamma || (v.total_off > 0 && (!A || !B || !rd || !r))) return SSPCG_ERR_INVALID_ARG;
-  const int per = kkt_per(v.nprob, v.max_N);
-  form_gamma_kernel<<<(unsigned)v.nprob * per, kKktThreads, 0, (cudaStream_t)stream>>>(v.ps, per, A, B, qd, rd, c, q, r,
+  const ChunkSplit split = kkt_split(v.nprob, v.max_N, v.max_nx, v.max_nu);
+  form_gamma_kernel<<<(unsigned)v.nprob * split.per, kKktThreads, 0, (cudaStream_t)stream>>>(v.ps, split, A, B, qd, rd, c, q, r,
                                                                                        gamma);
   KKT_CUDA(cudaGetLastError());
   return SSPCG_OK;
@@ -189,8 +187,8 @@ sspcg_status sspcg_recover_step_batched(sspcg_plan *plan, const float *A, const 
   const host::PlanView v = host::plan_view(plan);
   if (v.nprob == 0) return SSPCG_OK;
   if (!qd || !q || !mu || !dx || (v.total_off > 0 && (!A || !B || !rd || !r || !du))) return SSPCG_ERR_INVALID_ARG;
-  const int per = kkt_per(v.nprob, v.max_N);
-  recover_step_kernel<<<(unsigned)v.nprob * per, kKktThreads, 0, (cudaStream_t)stream>>>(v.ps, per, A, B, qd, rd, q, r,
+  const ChunkSplit split = kkt_split(v.nprob, v.max_N, v.max_nx, v.max_nu);
+  recover_step_kernel<<<(unsigned)v.nprob * split.per, kKktThreads, 0, (cudaStream_t)stream>>>(v.ps, split, A, B, qd, rd, q, r,
                                                                                          mu, dx, du);
   KKT_CUDA(cudaGetLastError());
   return SSPCG_OK;
