@@ -229,6 +229,7 @@ struct sspcg_plan {
   int64_t sizes[SSPCG_NUM_ARRAYS] = {};
   ProbDesc *d_desc = nullptr;
   int2 *d_kref = nullptr;  // (problem, block row) per knot
+  int2 *d_oref = nullptr;  // the same per off-diagonal block, for few_small_offs only
   int32_t *d_order = nullptr;  // problems, those with the most matrix entries first
   int64_t total_knots = 0, total_off = 0;
   std::vector<int64_t> knot_start;      // first knot (index into d_kref) of each problem, nprob + 1 entries
@@ -290,7 +291,7 @@ namespace {
 void plan_free(sspcg_plan *p) {
   if (!p) return;
   if (p->graph) cudaGraphExecDestroy(p->graph);
-  for (void *ptr : {(void *)p->d_desc, (void *)p->d_kref, (void *)p->d_order, (void *)p->d_knot_start, (void *)p->d_tdesc,
+  for (void *ptr : {(void *)p->d_desc, (void *)p->d_kref, (void *)p->d_oref, (void *)p->d_order, (void *)p->d_knot_start, (void *)p->d_tdesc,
                     (void *)p->d_tkref, (void *)p->d_toref, (void *)p->D64, (void *)p->E64,
                     (void *)p->PD64, (void *)p->PE64, (void *)p->d_work, (void *)p->d_counters, (void *)p->d_scratch, (void *)p->hbuf,
                     (void *)p->hint, (void *)p->hdbl, (void *)p->d_pad, (void *)p->d_pad_off, (void *)p->d_pad_list})
@@ -663,7 +664,7 @@ sspcg_status sspcg_build_schur(int32_t N, int32_t nx, int32_t nu, const float *A
   if (!shape_ok(N, nx, nu)) return SSPCG_ERR_INVALID_ARG;
   if (!qd || !D || (N > 0 && (!A || !rd || !E || (nu > 0 && !B)))) return SSPCG_ERR_INVALID_ARG;
   ProbSet ps{nullptr, single_desc(N, nx, nu), 1};
-  SSPCG_CUDA(launch_schur_f32(ps, N, nx, nu, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
+  SSPCG_CUDA(launch_schur_f32(ps, nullptr, N + 1, N, nx, nu, A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
   return SSPCG_OK;
 }
 
@@ -698,7 +699,7 @@ sspcg_status sspcg_build_precond(int32_t N, int32_t nx, sspcg_precond kind, cons
   ProbSet ps{nullptr, single_desc(N, nx, 0), 1};
   SSPCG_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
   SSPCG_CUDA(launch_precond_inv<float>(ps, nullptr, N + 1, nx, (int)kind, D, PD, status, st));
-  SSPCG_CUDA(launch_precond_off_f32(ps, N, nx, (int)kind, E, PD, PE, st, device_sms(), (int64_t)N * nx * nx));
+  SSPCG_CUDA(launch_precond_off_f32(ps, nullptr, N, N, nx, (int)kind, E, PD, PE, st, device_sms(), (int64_t)N * nx * nx));
   return SSPCG_OK;
 }
 
@@ -839,6 +840,9 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     cudaError_t e;
     if ((e = upload(&p->d_desc, p->hdesc)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = upload(&p->d_kref, row_refs(p->hdesc, 0))) != cudaSuccess) return fail(cuda_fail(e));
+    if (few_small_offs(p->total_off, p->max_nx) &&
+        (e = upload(&p->d_oref, row_refs(p->hdesc, 1))) != cudaSuccess)
+      return fail(cuda_fail(e));
     if ((e = upload(&p->d_knot_start, p->knot_start)) != cudaSuccess) return fail(cuda_fail(e));
     std::vector<int32_t> order(all);
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
@@ -986,8 +990,8 @@ sspcg_status sspcg_build_schur_batched(sspcg_plan *plan, const float *A, const f
   if (plan->nprob == 0) return SSPCG_OK;
   if (!qd || !D || !aligned16(qd) || !aligned16(D)) return SSPCG_ERR_INVALID_ARG;
   if (plan->total_off > 0 && (!A || !rd || !E || !B)) return SSPCG_ERR_INVALID_ARG;
-  SSPCG_CUDA(launch_schur_f32(plan_set(plan), plan->max_N, plan->max_nx, plan->max_nu, A, B, qd, rd, D, E,
-                              (cudaStream_t)stream, device_sms()));
+  SSPCG_CUDA(launch_schur_f32(plan_set(plan), plan->d_kref, plan->total_knots, plan->max_N, plan->max_nx, plan->max_nu,
+                              A, B, qd, rd, D, E, (cudaStream_t)stream, device_sms()));
   return SSPCG_OK;
 }
 
@@ -1076,8 +1080,8 @@ sspcg_status sspcg_build_precond_batched(sspcg_plan *plan, sspcg_precond kind, c
   for (const NxGroup &g : plan->nxg_all)
     SSPCG_CUDA(launch_precond_inv<float>(ProbSet{g.d_desc, ProbDesc{}, g.nprob}, g.d_refs, g.knots, g.nx,
                                          (int)kind, D, PD, status, st));
-  SSPCG_CUDA(launch_precond_off_f32(plan_set(plan), plan->max_N, plan->max_nx, (int)kind, E, PD, PE, st,
-                                    device_sms(), plan->sizes[SSPCG_ARRAY_OFF]));
+  SSPCG_CUDA(launch_precond_off_f32(plan_set(plan), plan->d_oref, plan->total_off, plan->max_N, plan->max_nx,
+                                    (int)kind, E, PD, PE, st, device_sms(), plan->sizes[SSPCG_ARRAY_OFF]));
   return SSPCG_OK;
 }
 

@@ -2,7 +2,7 @@
 // Sec. III, Sec. IV, Eq. jacobi).  One warp per knot; the batch is a flat
 // list of knots whose (problem, block row) pairs the plan tabulates.  The FP32
 // Schur blocks of diagonal costs and FP32 off-diagonal blocks are in
-// build_f32.cu; here these two run for the FP64 path.
+// build_f32.cu; here these two run for the FP64 path and for a few small blocks.
 #include <algorithm>
 #include <type_traits>
 
@@ -534,6 +534,9 @@ cudaError_t launch_precond_off(const ProbSet &ps, const int2 *refs, int64_t tota
   return cudaGetLastError();
 }
 
+template cudaError_t launch_schur_build<float>(const ProbSet &, const int2 *, int64_t, const float *, const float *,
+                                               const float *, const float *, float *, float *, cudaStream_t, int,
+                                               int);
 template cudaError_t launch_schur_build<double>(const ProbSet &, const int2 *, int64_t, const float *,
                                                 const float *, const float *, const float *, double *, double *,
                                                 cudaStream_t, int, int);
@@ -541,6 +544,8 @@ template cudaError_t launch_precond_inv<float>(const ProbSet &, const int2 *, in
                                                float *, int32_t *, cudaStream_t);
 template cudaError_t launch_precond_inv<double>(const ProbSet &, const int2 *, int64_t, int, int, const double *,
                                                 double *, int32_t *, cudaStream_t);
+template cudaError_t launch_precond_off<float>(const ProbSet &, const int2 *, int64_t, int, const float *,
+                                               const float *, float *, cudaStream_t, int, int64_t, int);
 template cudaError_t launch_precond_off<double>(const ProbSet &, const int2 *, int64_t, int, const double *,
                                                 const double *, double *, cudaStream_t, int, int64_t, int);
 

@@ -191,19 +191,33 @@ __global__ void __launch_bounds__(kOffThreads, 4) precond_off_f32_kernel(ProbSet
 
 }  // namespace
 
-cudaError_t launch_schur_f32(const ProbSet &ps, int max_N, int max_nx, int max_nu, const float *A,
-                             const float *B, const float *qd, const float *rd, float *D, float *E, cudaStream_t st, int sms) {
+// A CTA's barriers and index arithmetic take a microsecond that a few small blocks don't have: they stay with the warp
+// per knot of build.cu.  Schur blocks up to 4,500 knots: 3.1 us for 3.7 (nx 2, N 8 alone) and 4.3 for 4.8 (nx 2, 64
+// problems of N 64), but 128 of N 40, nx 4 5.2 by chunks for 6.2, one of N 8, nx 12 4.8 for 6.2.  Off-diagonal blocks up
+// to 8,000, us with the inverses: nx 2, N 64 alone 8.4 for 10.4, nx 3, 128 of N 40 12.5 for 13.9, 512 of N 20 14.5 either
+// way.
+bool few_small_knots(int64_t total, int max_nx, int max_nu) { return total <= 4500 && max_nx <= 8 && max_nu <= 8; }
+bool few_small_offs(int64_t total, int max_nx) { return total <= 8000 && max_nx <= 8; }
+
+cudaError_t launch_schur_f32(const ProbSet &ps, const int2 *refs, int64_t total_knots, int max_N, int max_nx, int max_nu,
+                             const float *A, const float *B, const float *qd, const float *rd, float *D, float *E,
+                             cudaStream_t st, int sms) {
   if (ps.nprob == 0) return cudaSuccess;
+  if (few_small_knots(total_knots, max_nx, max_nu))
+    return launch_schur_build<float>(ps, refs, total_knots, A, B, qd, rd, D, E, st, sms, std::max(max_nx, max_nu));
   const ChunkSplit split = chunk_split(ps.nprob, sms, max_N, schur_chunk(max_nx, max_nu), 3);
   schur_f32_kernel<<<(unsigned)ps.nprob * split.per, kSchurThreads, 0, st>>>(ps, split, A, B, qd, rd, D, E);
   return cudaGetLastError();
 }
 
-cudaError_t launch_precond_off_f32(const ProbSet &ps, int max_N, int max_nx, int kind, const float *E,
-                                   const float *PD, float *PE, cudaStream_t st, int sms, int64_t off_elems) {
+cudaError_t launch_precond_off_f32(const ProbSet &ps, const int2 *refs, int64_t total_off, int max_N, int max_nx,
+                                   int kind, const float *E, const float *PD, float *PE, cudaStream_t st, int sms,
+                                   int64_t off_elems) {
   if (off_elems == 0 || max_N == 0) return cudaSuccess;
   if (kind == 2 || kind == 3)  // block-Jacobi, Jacobi: no off-diagonal blocks
     return cudaMemsetAsync(PE, 0, sizeof(float) * off_elems, st);
+  if (few_small_offs(total_off, max_nx))
+    return launch_precond_off<float>(ps, refs, total_off, kind, E, PD, PE, st, sms, off_elems, max_nx);
   const ChunkSplit split = chunk_split(ps.nprob, sms, max_N, off_chunk(max_nx), 3);
   precond_off_f32_kernel<<<(unsigned)ps.nprob * split.per, kOffThreads, 0, st>>>(ps, split, kind == 0 ? 1.0f : 0.5f, E,
                                                                                  PD, PE);

@@ -203,19 +203,22 @@ inline bool pcg_one_ok(int op, bool f64, int red, int poly, int cg, int block, i
          pcg_one_layout(op, (int)N, nx, nu).total * (int64_t)sizeof(float) <= budget;
 }
 
-// Schur build and preconditioner assembly; Real = double (the FP64 path), for
-// the inverses also float (FP32 blocks).  refs[i] = (problem, block row) of work item i
+// Schur build and preconditioner assembly; Real = float (FP32 blocks; the Schur
+// and the off-diagonal blocks of few small knots only) or double (the FP64
+// path).  refs[i] = (problem, block row) of work item i
 // (nullptr: one problem, item i is block row i, or i + 1 for off-diagonals).
 // mx: the largest nx and nu of the launch (sizes the per-warp shared memory).
 template <typename Real>
 cudaError_t launch_schur_build(const ProbSet &ps, const int2 *refs, int64_t total_knots, const float *A,
                                const float *B, const float *qd, const float *rd, Real *D, Real *E,
                                cudaStream_t st, int sms, int mx);
-// The same in FP32 (build_f32.cu); max_N, max_nx, max_nu: the largest sizes of the set; off_elems: values of PE.
-cudaError_t launch_schur_f32(const ProbSet &ps, int max_N, int max_nx, int max_nu, const float *A, const float *B,
-                             const float *qd, const float *rd, float *D, float *E, cudaStream_t st, int sms);
-cudaError_t launch_precond_off_f32(const ProbSet &ps, int max_N, int max_nx, int kind, const float *E, const float *PD,
-                                   float *PE, cudaStream_t st, int sms, int64_t off_elems);
+// The same in FP32 (build_f32.cu), refs as above (read for few small knots only); max_N, max_nx, max_nu: the largest
+// sizes of the set; off_elems: values of PE.
+bool few_small_offs(int64_t total, int max_nx);
+cudaError_t launch_schur_f32(const ProbSet &ps, const int2 *refs, int64_t total_knots, int max_N, int max_nx, int max_nu,
+                             const float *A, const float *B, const float *qd, const float *rd, float *D, float *E, cudaStream_t st, int sms);
+cudaError_t launch_precond_off_f32(const ProbSet &ps, const int2 *refs, int64_t total_off, int max_N, int max_nx,
+                                   int kind, const float *E, const float *PD, float *PE, cudaStream_t st, int sms, int64_t off_elems);
 // Schur blocks with full SPD cost blocks from their inverses: Qi laid out like
 // D, R_{k-1}^-1 of problem p at roff[p] + (k-1) nu^2 (roff nullptr: offset 0).
 cudaError_t launch_schur_full(const ProbSet &ps, const int2 *refs, int64_t total_knots, const int64_t *roff,
