@@ -231,7 +231,7 @@ struct sspcg_plan {
   int2 *d_kref = nullptr;  // (problem, block row) per knot
   int2 *d_oref = nullptr;  // the same per off-diagonal block, for few_small_offs only
   int32_t *d_order = nullptr;  // problems, those with the most matrix entries first
-  int64_t total_knots = 0, total_off = 0;
+  int64_t total_knots = 0, total_off = 0, total_rows = 0;
   std::vector<int64_t> knot_start;      // first knot (index into d_kref) of each problem, nprob + 1 entries
   int64_t *d_knot_start = nullptr;
   // FP64 subset: descriptors whose odiag/ooff point into plan-owned FP64 blocks
@@ -808,6 +808,7 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     all.push_back(i);
     p->mx = std::max(p->mx, std::max(nx[i], nu[i]));
     p->max_nx = std::max(p->max_nx, nx[i]);
+    p->total_rows += (int64_t)(N[i] + 1) * nx[i];
     p->max_nu = std::max(p->max_nu, nu[i]);
     p->max_N = std::max(p->max_N, N[i]);
     const bool f64 = opts->precision == SSPCG_PRECISION_F64 ||
@@ -1614,6 +1615,7 @@ PlanView plan_view(const sspcg_plan *p) {
   v.d_knot_start = p->d_knot_start;
   v.total_off = p->total_off;
   v.max_nx = p->max_nx;
+  v.rows = p->total_rows;
   v.max_nu = p->max_nu;
   v.max_N = p->max_N;
   return v;

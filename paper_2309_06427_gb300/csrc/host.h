@@ -19,6 +19,7 @@ struct PlanView {
   const int64_t *d_knot_start;  // the same on the device
   int64_t total_off;            // number of off-diagonal blocks
   int32_t max_nx, max_nu, max_N;  // largest nx, nu and N of the batch
+  int64_t rows;                   // rows of all problems
 };
 
 int sms();
