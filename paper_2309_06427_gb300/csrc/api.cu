@@ -221,6 +221,7 @@ struct sspcg_plan {
   int32_t nprob = 0;
   int mx = 1;       // largest nx and nu of the batch
   int32_t max_nx = 1, max_nu = 0, max_N = 0;
+  bool wide = false;  // some nu > nx
   int mx_tiny = 1;  // of its FP64 subset
   std::vector<NxGroup> nxg_all, nxg_tiny;
   sspcg_options opts{};
@@ -764,7 +765,7 @@ sspcg_status sspcg_residual_qp(int32_t N, int32_t nx, int32_t nu, const float *A
   if (!shape_ok(N, nx, nu) || !qd || !gamma || !lambda || !relres_true) return SSPCG_ERR_INVALID_ARG;
   if (N > 0 && (!A || !rd || (nu > 0 && !B))) return SSPCG_ERR_INVALID_ARG;
   ProbSet ps{nullptr, single_desc(N, nx, nu), 1};
-  SSPCG_CUDA(launch_residual_qp(ps, nullptr, A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
+  SSPCG_CUDA(launch_residual_qp(ps, nullptr, nu > nx, A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
   return SSPCG_OK;
 }
 
@@ -808,6 +809,7 @@ sspcg_status sspcg_plan_create(sspcg_plan **plan, int32_t nprob, const int32_t *
     all.push_back(i);
     p->mx = std::max(p->mx, std::max(nx[i], nu[i]));
     p->max_nx = std::max(p->max_nx, nx[i]);
+    p->wide = p->wide || nu[i] > nx[i];
     p->total_rows += (int64_t)(N[i] + 1) * nx[i];
     p->max_nu = std::max(p->max_nu, nu[i]);
     p->max_N = std::max(p->max_N, N[i]);
@@ -1165,7 +1167,8 @@ sspcg_status sspcg_residual_qp_batched(sspcg_plan *plan, const float *A, const f
   if (plan->nprob == 0) return SSPCG_OK;
   if (!qd || !gamma || !lambda || !relres_true || (plan->total_off > 0 && (!A || !B || !rd)))
     return SSPCG_ERR_INVALID_ARG;
-  SSPCG_CUDA(launch_residual_qp(plan_set(plan), plan->d_order, A, B, qd, rd, gamma, lambda, relres_true, (cudaStream_t)stream));
+  SSPCG_CUDA(launch_residual_qp(plan_set(plan), plan->d_order, plan->wide, A, B, qd, rd, gamma, lambda, relres_true,
+                                (cudaStream_t)stream));
   return SSPCG_OK;
 }
 

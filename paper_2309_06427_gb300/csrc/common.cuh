@@ -144,6 +144,17 @@ __host__ __device__ __forceinline__ int chunk_rows(int nx, int nu) {
   return c > 64 ? 64 : c;
 }
 
+// Chunks of the true residual (residual.cu), which keeps nx + nu doubles per block row beside the blocks, in
+// kResFloats, for batches with some nu > nx: as above, but at least 128 rows where they fit, so that the half that works
+// row by row has a warp for every quarter of the SM (N 64 to 512 alone: nx 4, nu 28 1.9 times as fast, nx 1, nu 28 3
+// times).
+constexpr int kResFloats = kChunkFloats + 2 * (kChunkItems + kMaxNx);
+__host__ __device__ __forceinline__ int residual_rows(int nx, int nu) {
+  const int fit = kResFloats / (nx * (nx | 1) + nx * (nu | 1) + 2 * (nx + nu)), few = (128 + nx - 1) / nx;
+  const int c = chunk_rows(nx, nu), w = few < fit ? few : fit;
+  return c > w ? c : w > 64 ? 64 : w;
+}
+
 // CTAs of a launch over chunks: ``per`` for every problem, which is cut into ``share`` chunks at least.
 struct ChunkSplit {
   int per, share;

@@ -234,8 +234,8 @@ template <typename Real>
 cudaError_t launch_precond_off(const ProbSet &ps, const int2 *refs, int64_t total_off, int kind,
                                const Real *E, const Real *PD, Real *PE, cudaStream_t st, int sms, int64_t off_elems,
                                int mx);
-// order: problem indices in the order in which they start (device), or nullptr: as numbered.
-cudaError_t launch_residual_qp(const ProbSet &ps, const int32_t *order, const float *A, const float *B, const float *qd,
+// order: problem indices in the order in which they start (device), or nullptr: as numbered; wide: some nu > nx.
+cudaError_t launch_residual_qp(const ProbSet &ps, const int32_t *order, bool wide, const float *A, const float *B, const float *qd,
                                const float *rd, const float *gamma, const float *lambda, double *relres_true,
                                cudaStream_t st);
 

@@ -46,6 +46,9 @@ __device__ __forceinline__ double divide(double s, float q) {
   return fma(fma(-d, t, s), y, t);
 }
 
+// WIDE: chunks of residual_rows, v_x and v_u before the blocks; otherwise of chunk_rows, with ten registers less
+// and so one CTA more to an SM.
+template <bool WIDE>
 __global__ void __launch_bounds__(kResThreads) residual_qp_kernel(ProbSet ps, const int32_t *order,
                                                                   const float *__restrict__ A,
                                                                   const float *__restrict__ B,
@@ -53,20 +56,21 @@ __global__ void __launch_bounds__(kResThreads) residual_qp_kernel(ProbSet ps, co
                                                                   const float *__restrict__ rd,
                                                                   const float *__restrict__ gamma,
                                                                   const float *__restrict__ lambda, double *out) {
-  __shared__ float sm[kChunkFloats];
+  __shared__ __align__(16) float sm[WIDE ? kResFloats : kChunkFloats];
   __shared__ double sx[kChunkItems + 2 * kMaxNx];  // lambda of the chunk's block rows and of the next one
-  __shared__ double sv[kChunkItems + kMaxNx];      // v_x and v_u of the chunk, nx + nu per block row
+  __shared__ double sv_[WIDE ? 1 : kChunkItems + kMaxNx];
   __shared__ double sy[kMaxNx];                    // A_{k-1} v_x(k-1) + B_{k-1} v_u(k-1) for the next chunk's first row
   __shared__ double red[2][kResThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int p = blockIdx.x; p < ps.nprob; p += gridDim.x) {
     const ProbDesc d = ps.get(order ? order[p] : p);
-    const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu, C = chunk_rows(nx, nu);
+    const int N = d.N, nx = d.nx, nu = d.nu, m = nx + nu, C = WIDE ? residual_rows(nx, nu) : chunk_rows(nx, nu);
     const int lda = nx | 1, ldb = nu | 1;
     const float *Ap = A + d.oA, *Bp = B + d.oB, *q = qd + d.oq, *r = rd + d.orr;
     const float *g = gamma + d.ovec, *x = lambda + d.ovec;
     const Divisor by_m(m), by_nx(nx);
-    float *sA = sm, *sB = sm + C * nx * lda;
+    double *sv = WIDE ? reinterpret_cast<double *>(sm) : sv_;  // v_x and v_u of the chunk, nx + nu per block row
+    float *sA = WIDE ? sm + 2 * C * m : sm, *sB = sA + C * nx * lda;
     double res2 = 0.0, g2 = 0.0;
     if (tid < nx) sy[tid] = 0.0;
     for (int k0 = 0; k0 <= N; k0 += C) {
@@ -133,11 +137,14 @@ __global__ void __launch_bounds__(kResThreads) residual_qp_kernel(ProbSet ps, co
   }
 }
 
-cudaError_t launch_residual_qp(const ProbSet &ps, const int32_t *order, const float *A, const float *B, const float *qd,
+cudaError_t launch_residual_qp(const ProbSet &ps, const int32_t *order, bool wide, const float *A, const float *B, const float *qd,
                                const float *rd, const float *gamma, const float *lambda, double *relres_true,
                                cudaStream_t st) {
   if (ps.nprob == 0) return cudaSuccess;
-  residual_qp_kernel<<<ps.nprob, kResThreads, 0, st>>>(ps, order, A, B, qd, rd, gamma, lambda, relres_true);
+  if (wide)
+    residual_qp_kernel<true><<<ps.nprob, kResThreads, 0, st>>>(ps, order, A, B, qd, rd, gamma, lambda, relres_true);
+  else
+    residual_qp_kernel<false><<<ps.nprob, kResThreads, 0, st>>>(ps, order, A, B, qd, rd, gamma, lambda, relres_true);
   return cudaGetLastError();
 }
 
