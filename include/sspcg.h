@@ -522,8 +522,9 @@ sspcg_status sspcg_plan_join(sspcg_plan *plan, sspcg_stream stream);
  * the work order travel as the parameter block of one set-up kernel (the
  * driver copies launch parameters when it records the launch), which writes
  * the descriptors into the array and clears the queue counters and
- * ``status`` on ``stream``; then one PCG launch per nx follows.  The call
- * returns without waiting for the GPU.
+ * ``status`` on ``stream``; then one PCG launch per nx follows: the row-pair
+ * kernel (see sspcg_plan_create) when every problem of that nx fits it, the
+ * general one otherwise.  The call returns without waiting for the GPU.
  *
  * Warm-up: the first call on a device looks up the array's device address
  * (cudaGetSymbolAddress); make it before any stream capture.  Later calls
@@ -531,7 +532,8 @@ sspcg_status sspcg_plan_join(sspcg_plan *plan, sspcg_stream stream);
  * solves the captured batch again (same shapes and pointers).  The first
  * launch of each PCG kernel variant (each nx and each reduction, schedule or
  * CG option) sets that kernel's shared-memory attribute and, under lazy
- * module loading, may load its code.  Callers with a time bound (a control
+ * module loading, may load its code; of the two kernels that horizons choose
+ * between, the first call with an nx loads both.  Callers with a time bound (a control
  * loop) should make one call per nx and option set they will use before the
  * loop starts; later calls do neither.
  */

@@ -151,6 +151,26 @@ sspcg_status scratch_address(NoAllocScratch **out) {
   return SSPCG_OK;
 }
 
+std::atomic<uint32_t> g_loaded[kMaxDevices];  // bit nx: load_both has run
+
+// The horizons of a call decide between two kernels of one nx (a thread per row pair, or the general one): the first
+// call with that nx loads both and sets their shared-memory attributes, so that a later one of other horizons does
+// neither.
+cudaError_t load_both(int nx) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint32_t bit = 1u << nx;
+  if (g_loaded[dev].load(std::memory_order_acquire) & bit) return cudaSuccess;
+  int ctas = 0;
+  for (bool one : {true, false}) {
+    e = occupancy_pcg(nx, kOpQp, kRedDf, false, false, false, false, one, 64, 0, &ctas);
+    if (e != cudaSuccess) return e;
+  }
+  g_loaded[dev].fetch_or(bit, std::memory_order_acq_rel);
+  return cudaSuccess;
+}
+
 }  // namespace
 
 extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int32_t *N, const int32_t *nx,
@@ -178,7 +198,8 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
   struct Group {
     int32_t count = 0, first = 0;
     int64_t rows = 0, smem = 0, maxN = 0, smem_one = 0;
-    bool one = true;  // every problem of the group runs with a thread per row pair
+    bool one = true;  // every problem of the group runs with a thread per row pair; one that doesn't fit that kernel
+                      // sends all of its nx to the general one
   } groups[kMaxNx + 1];
   for (int32_t i = 0; i < nprob; ++i) {
     s.N[i] = (int16_t)N[i];
@@ -250,6 +271,7 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
     ga.nwork = g.count;
     ga.counter = scr->counters + counter++;
     ga.one = g.one ? 1 : 0;
+    if (host::fits_one(kOpQp, opts, 0, m, 0) && (e = load_both(m)) != cudaSuccess) return host::cuda_error(e);
     e = launch_pcg(m, kOpQp, host::reduction_mode(opts->reduction), false, ga, grid, block, (size_t)smem, st);
     if (e != cudaSuccess) return host::cuda_error(e);
   }
