@@ -88,9 +88,16 @@ int auto_block(int64_t rows) {
 int one_block(int64_t N, int nx) { return (int)std::max<int64_t>(64, round_up((N + 1) * tile_half(nx), 32)); }
 
 // Whether a problem runs with a thread per row pair: a solve of these options, not streaming by request, that fits
-// whole with at most 512 pairs (the registers of a thread allow no more).  Measured faster at every size it takes,
-// from 1.4x (nx = 14, N = 64) to 1.8x (nx = 4, N = 64); the line lies at what fits.
-bool one_fits(int op, const sspcg_options *o, bool f64, int64_t N, int nx, int nu) {
+// whole with at most 512 pairs (the registers of a thread allow no more); same: problems of that nx in the call.
+// Measured over nx 1 to 28, N from 4 to the most that fits, nu = ceil(nx / 2) and 28, 1 and 304 problems: QP form 1.0
+// (nx 8, nu 28, N 4) to 2.6 times (nx 1, nu 28, N 100) as fast as the general kernel, 1.4 on average (nx 14, N 64 1.35, nx
+// 4, N 64 1.5); block form 1.1 to 1.8.  Only where half or a sixth of the pairs' rows are padding (nx 1 and 5) do many
+// long problems lose: 304 of nx 1, N 511 307 us for 274, 1520 of N 383 1,163 for 876, of nx 5, N 169 1,993 for 1,840 (N
+// 120 1,219 for 1,277).
+bool one_fits(int op, const sspcg_options *o, bool f64, int64_t N, int nx, int nu, int64_t same) {
+  const int64_t sms = device_sms();
+  if (nx == 1 && ((same > sms && N > 320) || (same > 2 * sms && N > 64))) return false;
+  if (nx == 5 && same > 2 * sms && N > 140) return false;
   return o->schedule != SSPCG_SCHED_STREAM &&
          pcg_one_ok(op, f64, red_mode(o->reduction), o->poly_degree, o->cg_variant,
                     o->block_threads > 0 ? o->block_threads : 512, smem_budget(), N, nx, nu);
@@ -149,7 +156,9 @@ int sms() { return device_sms(); }
 int reduction_mode(int32_t r) { return red_mode(r); }
 int block_for_rows(int64_t rows) { return auto_block(rows); }
 int block_for_pairs(int64_t N, int nx) { return one_block(N, nx); }
-bool fits_one(int op, const sspcg_options *o, int64_t N, int nx, int nu) { return one_fits(op, o, false, N, nx, nu); }
+bool fits_one(int op, const sspcg_options *o, int64_t N, int nx, int nu, int64_t same) {
+  return one_fits(op, o, false, N, nx, nu, same);
+}
 bool fit(int op, int sched, int N, int nx, int nu, bool f64, int poly, int cg, int *K, int64_t *bytes) {
   return pcg_fit(op, sched, N, nx, nu, f64, poly, cg, K, bytes);
 }
@@ -435,10 +444,12 @@ sspcg_status plan_groups(sspcg_plan *p, GroupSet &set, const std::vector<ProbDes
   std::vector<std::vector<int32_t>> buckets(kKinds * kClasses * (kMaxNx + 1));
   std::vector<int64_t> bytes(descs.size(), 0);
   const int64_t budget = smem_budget();
+  std::vector<int64_t> same(kMaxNx + 1, 0);
+  for (int32_t i : members) ++same[descs[i].nx];
   for (int32_t i : members) {
     const ProbDesc &d = descs[i];
     int K = 0;
-    const bool one = one_fits(set.op, &p->opts, set.f64, d.N, d.nx, d.nu);
+    const bool one = one_fits(set.op, &p->opts, set.f64, d.N, d.nx, d.nu, same[d.nx]);
     int kind = one ? 1 : 0;
     if (one) {
       if (p->opts.schedule == SSPCG_SCHED_WARP && set.op == kOpQp &&
@@ -716,7 +727,7 @@ static sspcg_status solve_single(int op, bool f64, int32_t N, int32_t nx, int32_
   if (op == kOpBlock && (!D || (N > 0 && !E))) return SSPCG_ERR_INVALID_ARG;
   int K = 0;
   int64_t bytes = 0;
-  const bool one = one_fits(op, opts, f64, N, nx, nu);
+  const bool one = one_fits(op, opts, f64, N, nx, nu, 1);
   if (one) bytes = pcg_one_layout(op, N, nx, nu).total * (int64_t)sizeof(float);
   else if (!pcg_fit(op, opts->schedule, N, nx, nu, f64, opts->poly_degree, opts->cg_variant, &K, &bytes))
     return SSPCG_ERR_UNSUPPORTED;

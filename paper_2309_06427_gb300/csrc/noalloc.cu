@@ -25,7 +25,7 @@ int sms();
 int reduction_mode(int32_t r);
 int block_for_rows(int64_t rows);
 int block_for_pairs(int64_t N, int nx);
-bool fits_one(int op, const sspcg_options *o, int64_t N, int nx, int nu);
+bool fits_one(int op, const sspcg_options *o, int64_t N, int nx, int nu, int64_t same);
 bool fit(int op, int sched, int N, int nx, int nu, bool f64, int poly, int cg, int *K, int64_t *bytes);
 sspcg_status check_options(const sspcg_options *o);
 bool valid_shape(int N, int nx, int nu);
@@ -201,6 +201,7 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
     bool one = true;  // every problem of the group runs with a thread per row pair; one that doesn't fit that kernel
                       // sends all of its nx to the general one
   } groups[kMaxNx + 1];
+  for (int32_t i = 0; i < nprob; ++i) ++groups[nx[i]].count;
   for (int32_t i = 0; i < nprob; ++i) {
     s.N[i] = (int16_t)N[i];
     s.nx[i] = (uint8_t)nx[i];
@@ -208,7 +209,7 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
     int K = 0;
     int64_t bytes = 0;
     Group &g = groups[nx[i]];
-    const bool one = host::fits_one(kOpQp, opts, N[i], nx[i], nu[i]);
+    const bool one = host::fits_one(kOpQp, opts, N[i], nx[i], nu[i], g.count);
     if (!host::fit(kOpQp, opts->schedule, N[i], nx[i], nu[i], false, opts->poly_degree, opts->cg_variant, &K,
                    &bytes))
       return SSPCG_ERR_UNSUPPORTED;
@@ -216,7 +217,6 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
     if (one)
       g.smem_one = std::max(g.smem_one, pcg_one_layout(kOpQp, N[i], nx[i], nu[i]).total * (int64_t)sizeof(float));
     g.maxN = std::max<int64_t>(g.maxN, N[i]);
-    ++g.count;
     g.rows = std::max<int64_t>(g.rows, (int64_t)(N[i] + 1) * nx[i]);
     g.smem = std::max<int64_t>(g.smem, bytes);
   }
@@ -271,7 +271,7 @@ extern "C" sspcg_status sspcg_solve_qp_batched_noalloc(int32_t nprob, const int3
     ga.nwork = g.count;
     ga.counter = scr->counters + counter++;
     ga.one = g.one ? 1 : 0;
-    if (host::fits_one(kOpQp, opts, 0, m, 0) && (e = load_both(m)) != cudaSuccess) return host::cuda_error(e);
+    if (host::fits_one(kOpQp, opts, 0, m, 0, 1) && (e = load_both(m)) != cudaSuccess) return host::cuda_error(e);
     e = launch_pcg(m, kOpQp, host::reduction_mode(opts->reduction), false, ga, grid, block, (size_t)smem, st);
     if (e != cudaSuccess) return host::cuda_error(e);
   }
