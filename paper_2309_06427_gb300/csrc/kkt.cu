@@ -200,13 +200,15 @@ struct Set {
   unsigned knot_ctas() const { return (unsigned)cdiv(knots, kKktWarps); }
 };
 
-// Chunks for the right-hand side: of small blocks (nx 8 on average, no more inputs than states) from 10,000 knots on, of
-// medium ones (16) from 60,000, never of large ones.  Chunks against warps, us, with A and B in L2 unless said otherwise:
-// nx 4, 64 problems of N 64 4.9 / 3.3, 512 of N 20 5.2 / 5.4, 8192 of N 20 33 / 51; nx 14, 2048 of N 20 25 / 20, 1024 of N
-// 64 40 / 40 (from HBM 53 / 56), 8192 of N 20 95 / 113; nx 21, 8192 of N 20 163 / 154; N 16-128, nx 4, 12, 14, 21: 512
-// problems 26 / 19 (from HBM 38 / 36), 4096 171 / 195.
+// Chunks for the right-hand side: of small blocks (nx 8 on average) from 10,000 knots on, 20,000 with more inputs than
+// states, of medium ones (16) from 60,000, never of large ones nor with more than 8 inputs and fewer states.  Chunks
+// against warps, us, with A and B in L2 unless said otherwise: nx 4, 64 problems of N 64 4.9 / 3.3, 512 of N 20 5.2 / 5.4,
+// 8192 of N 20 33 / 51; nx 1, nu 2, 1024 of N 64 12 / 20; nx 14, 2048 of N 20 25 / 20, 1024 of N 64 40 / 40 (from HBM 53 /
+// 56), 8192 of N 20 95 / 113; nx 21, 8192 of N 20 163 / 154; nx 4, nu 28, 1024 of N 64 38 / 34; N 16-128, nx 4, 12, 14, 21:
+// 512 problems 26 / 19 (from HBM 38 / 36), 4096 171 / 195.
 bool gamma_chunks(const Set &s) {
-  return (s.rows <= 8 * s.knots && s.max_nu <= s.max_nx && s.knots >= 10000) ||
+  if (s.max_nu > s.max_nx && s.max_nu > 8) return false;
+  return (s.rows <= 8 * s.knots && s.knots >= (s.max_nu > s.max_nx ? 20000 : 10000)) ||
          (s.rows <= 16 * s.knots && s.knots >= 60000);
 }
 // Chunks for the primal step from 16,000 knots on, unless there are more than two inputs to a state, and of large blocks
