@@ -37,13 +37,15 @@ PRECOND = "sym"
 SMEM_BYTES_PER_CLK_PER_SM = 128  # shared-memory bandwidth of one SM (32 banks x 4 B per clock)
 MLP_FLOP_PER_ROW = 2 * (1344 * 256 + 256 * 256 + 256 * 32)  # warm-start network forward, one knot row
 def kernel_source_hash() -> str:
-    """First 16 hex digits of the SHA-256 of the PCG kernel source (pcg.cuh, and its layout and arguments in
+    """First 16 hex digits of the SHA-256 of the PCG kernels' source (pcg*.cuh, and their layouts and arguments in
     kernels.h) with comments and blank space removed, so that only code changes alter it."""
+    import glob
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in ("pcg.cuh", "kernels.h"):
-        with open(os.path.join(ROOT, "paper_2309_06427_gb300", "csrc", f)) as fh:
+    csrc = os.path.join(ROOT, "paper_2309_06427_gb300", "csrc")
+    for f in sorted(glob.glob(os.path.join(csrc, "pcg*.cuh"))) + [os.path.join(csrc, "kernels.h")]:
+        with open(f) as fh:
             src = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         src = re.sub(r"//[^\n]*", "", src)
         h.update("".join(src.split()).encode())
@@ -959,7 +961,8 @@ def main():
                      "traffic_note": "DRAM bytes per PCG launch set of the batch (ncu, profiles/); the blocks are "
                                      "read from shared memory and L2, so HBM traffic is far below the "
                                      "algorithmic bytes",
-                     "kernel": "pcg_kernel (all FP32 PCG launches of the batch, timed alone)",
+                     "kernel": "pcg_one_kernel (problems that fit in shared memory whole) and pcg_kernel (the rest): "
+                               "all FP32 PCG launches of the batch, timed alone",
                      "peak_source": "measured: sspcg_measure_smem_bandwidth, conflict-free shared-memory reads "
                                     "on every SM (the better of 32-bit and 128-bit loads)",
                      "peak_measured_lds32_gbs": smem_4, "peak_measured_lds128_gbs": smem_16,

@@ -121,8 +121,8 @@ __device__ __forceinline__ T slot_sum(const T *slots, int l16, int nw, T zero) {
 }
 // In FP64 a butterfly over the next power of two of slots, repeated across the half: the steps that would only add
 // zeros change no bit, and an FP64 addition keeps its SM quarter's unit for 76 cycles whatever it adds (eight of them
-// per iteration and warp in CTAs of one warp; 16,384 problems, N 8-32, nx 2, 4, 6: 11.36 to 10.92 ms; nx 2, N 20 alone:
-// 102 to 96 us).  Double-float additions are cheap next to the branches: there the full butterfly stays.
+// per iteration and warp in CTAs of one warp; 16,384 problems, N 8-32, nx 2, 4, 6: 11.36 to 10.92 ms replayed on the same
+// values, 11.50 to 11.20 the first time on new ones; nx 2, N 20 alone: 102 to 96 us).  Double-float additions are cheap next to the branches: there the full butterfly stays.
 __device__ __forceinline__ double slot_sum(const double *slots, int l16, int nw, double zero) {
   const int span = nw > 8 ? 16 : nw > 4 ? 8 : nw > 2 ? 4 : nw;
   const int l = l16 & (span - 1);

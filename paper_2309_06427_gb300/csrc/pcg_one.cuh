@@ -26,10 +26,11 @@
 // pcg.cuh's, renormalised after every addition: folding the low parts only at
 // the end takes 5 % (nx = 14) to 15 % (nx = 4) less and leaves the sums 1.2
 // times (terms of one sign) to 1.9 times as far from the exact ones.
-// What bounds it: the shared-memory load pipe for the larger blocks (every
-// matrix entry comes through it once per use, a third of the tile loads by
-// columns with two-way bank conflicts where a warp phase crosses a block row),
-// the latency of five barriers and two block sums for the smaller ones.
+// What bounds it: the shared-memory load pipe for the larger blocks (nx = 14, 512
+// threads: 76 % busy; every matrix entry comes through it once per use, a quarter
+// of the wavefronts are bank conflicts of tile loads by columns where a warp phase
+// crosses a block row), the latency of five barriers and two block sums for the
+// smaller ones (nx = 4: a third of the issue slots and 28 % of L1 busy).
 #pragma once
 
 #include "pcg.cuh"
