@@ -235,8 +235,8 @@ cudaError_t launch_precond_off(const ProbSet &ps, const int2 *refs, int64_t tota
                                const Real *E, const Real *PD, Real *PE, cudaStream_t st, int sms, int64_t off_elems,
                                int mx);
 // order: problem indices in the order in which they start (device), or nullptr: as numbered; wide: some nu > nx.
-cudaError_t launch_residual_qp(const ProbSet &ps, const int32_t *order, bool wide, const float *A, const float *B, const float *qd,
-                               const float *rd, const float *gamma, const float *lambda, double *relres_true,
+cudaError_t launch_residual_qp(const ProbSet &ps, const int32_t *order, bool wide, const float *A, const float *B,
+                               const float *qd, const float *rd, const float *gamma, const float *lambda, double *relres_true,
                                cudaStream_t st);
 
 }  // namespace sspcg
