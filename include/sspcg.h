@@ -267,7 +267,8 @@ sspcg_status sspcg_residual_qp(int32_t N, int32_t nx, int32_t nu, const float *A
  * and picks a kernel schedule per problem class: FP32 problems that fit in
  * shared memory whole and have at most 512 pairs of rows take the row-pair
  * kernel (a thread per two adjacent rows; textbook PCG, double-float sums,
- * degree 0, any schedule but STREAM), the others the general kernel.  Both
+ * degree 0, any schedule but STREAM; of nx 1 and 5 only the shorter ones when
+ * there are many), the others the general kernel.  Both
  * form the same block products; their dot products group the same terms
  * differently, so results agree to rounding.  It also holds padded
  * copies of A, B and PE for the problems that do not fit in shared memory
