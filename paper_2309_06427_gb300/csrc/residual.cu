@@ -10,9 +10,9 @@
 // share one loop, so that a warp runs each FP64 instruction once for all its
 // lanes.  Problems go to the CTAs largest first: an SM holds several at a time,
 // and a large one begun late would outlast all others.  The call with the two
-// steps of kkt.cu, 4096 problems of N 20-100 and nx 4, 12, 14, 21: 2.47 ms before,
-// 1.49 ms in chunks in the order of the batch, 1.26 ms largest first
-// (1.36 ms with CTAs of 128 threads).
+// steps of kkt.cu, 4096 problems of N 16-128 and nx 4, 12, 14, 21: 2.47 ms before,
+// 1.49 ms in chunks in the order of the batch, 1.26 ms largest first (1.36 ms
+// with CTAs of 128 threads), 1.20 ms with the two steps as they are cut now.
 #include "common.cuh"
 #include "kernels.h"
 
